@@ -433,17 +433,20 @@ pttk_status pttk_batch_create(const pttk_tt* tt, int B, const int64_t* xoff, con
 void pttk_batch_free(pttk_batch* b);
 
 /* Launch configuration of the plan's tensor-core factor build; pttk_batch_get_config reports
- * the current one and how many exist (8). 0 (the default): the kernel that generates the A
- * operand in shared memory with four separate epilogue warps, which drain two alternating
- * tensor-memory accumulators while the next tile's products run (ranks whose two accumulators
- * or staging tiles do not fit fall back to configuration 1); 1 and 2: the same kernel without
+ * the current one and how many exist (8). 0 (the default): for the FP16/BF16 forms with d >= 2,
+ * the kernel on pairs of SMs (256 points a pair, A generated in tensor memory, each core chunk
+ * split over the two SMs); for the other forms, d = 1 and ranks it cannot hold, the kernel that
+ * generates the A operand in shared memory with four separate epilogue warps, which drain two
+ * alternating tensor-memory accumulators while the next tile's products run (ranks whose two
+ * accumulators or staging tiles do not fit fall back to configuration 1); 1 and 2: the latter without
  * the epilogue warps, with 128- or 64-byte chunks of K per row; 3, 4, 5: for the FP16/BF16
  * forms, the kernel that generates A in tensor memory and keeps the chain's intermediate in
  * registers, run in thread-block clusters of 1, 2 or 4 CTAs that share each core chunk by a
  * multicast copy (ranks it cannot hold fall back to configuration 1); 6: for the FP16/BF16
- * forms, A in tensor memory with the epilogue warps of configuration 0 and a B ring of 3-4
- * slots in the shared memory A no longer takes (ranks it cannot hold fall back to
- * configuration 0); 7: configuration 0 with 64-byte chunks of K per row in a ring of 4 slots. */
+ * forms, A in tensor memory with separate epilogue warps and a B ring of 3-4 slots in the
+ * shared memory A no longer takes (ranks it cannot hold fall back to the kernel with A in shared
+ * memory); 7: A in shared memory with epilogue warps, 64-byte chunks of K per row in a ring of 4
+ * slots. */
 pttk_status pttk_batch_set_config(pttk_batch* b, int cfg);
 pttk_status pttk_batch_get_config(const pttk_batch* b, int* cfg, int* n_configs);
 

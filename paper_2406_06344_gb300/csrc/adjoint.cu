@@ -290,9 +290,11 @@ pttk_status grad_typed(const pttk_tt* tt, const double* theta, const T* X, int64
     PTTK_TRY(factor_build_run(tt, true, X, N_s, prec, U, s));
     PTTK_TRY(factor_build_run(tt, false, Y, N_t, prec, V, s));
   } else {
+    // the shared-memory kernel: the theta-gradient is an FP64 result of these factors, and their last
+    // FP32 bits differ between the chain kernels
     PTTK_TRY(factor_build_tc(tt, tt_tc_cache(tt), reinterpret_cast<const float*>(X), N_s,
                              reinterpret_cast<const float*>(Y), N_t, prec, reinterpret_cast<float*>(U),
-                             reinterpret_cast<float*>(V), tt_status_word(tt), 0, s));
+                             reinterpret_cast<float*>(V), tt_status_word(tt), kTcSharedA, s));
   }
   PTTK_TRY(weighted_sum<T>(U, w, N_s, rs, a, partial, nparts, s));
   PTTK_TRY(weighted_sum<T>(V, z, N_t, rt, b, partial, nparts, s));

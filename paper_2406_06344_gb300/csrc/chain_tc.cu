@@ -37,9 +37,6 @@
 // Waits: every mbarrier wait is bounded; on timeout the CTA records PTTK_ETIMEOUT in a device
 // status word, stops issuing work, waits (bounded) for its outstanding copies and MMAs, frees
 // its TMEM and returns.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-#include <stdint.h>
 #include <stdio.h>
 
 #include <algorithm>
@@ -47,7 +44,9 @@
 #include <mutex>
 #include <vector>
 
+#include "chain_pair.cuh"
 #include "pttk_internal.cuh"
+#include "tcgen05.cuh"
 
 namespace pttk {
 
@@ -55,166 +54,6 @@ int oriented_core_dims(const pttk_tt* tt, bool source, int step, int* R_in, int*
 const void* oriented_core_ptr(const pttk_tt* tt, bool source, int k, bool fp64);
 
 namespace {
-
-constexpr int TILE_M = 128;
-
-// ---------------- PTX wrappers ------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void fence_mbar_init() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// try_wait with a suspend-time hint: the thread sleeps in hardware until the phase completes
-// or about `ns` nanoseconds have passed, whichever comes first (the completion wakes it at
-// once, so the hint costs no latency; it only spares the issue slots of repeated polls).
-__device__ __forceinline__ bool mbar_try_wait_hint(uint64_t* bar, uint32_t parity, uint32_t ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait for the completion of the phase with the given parity: gives up after ~2 s
-// (2^32 SM clocks, or 2^24 polls of up to 0.1 ms each) or as soon as another thread of the CTA
-// has raised the abort flag. Each poll suspends the thread in hardware until the phase
-// completes (or the hint runs out), so no software sleep adds a wake-up delay to a hand-off.
-__device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, const volatile int* abort_flag) {
-  const long long t0 = clock64();
-  for (uint32_t i = 0; i < (1u << 24); ++i) {
-    if (mbar_try_wait_hint(bar, parity, 100000u)) return true;
-    if (*abort_flag || clock64() - t0 > (4ll << 30)) return false;
-  }
-  return false;
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const volatile int* abort_flag) {
-  return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort_flag);
-}
-__device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)),
-               "r"(ncols)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-// 32 consecutive TMEM columns of this warp's 32 lanes (one row per thread).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-// 16 consecutive TMEM columns of this warp's 32 lanes (one row per thread).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-
-// UMMA shared-memory descriptor: no swizzle, K-major; K-adjacent core matrices 128 B apart
-// (leading byte offset), 8-row groups `sbo` bytes apart (stride byte offset).
-__device__ __forceinline__ uint64_t smem_desc2(uint32_t saddr, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((128u >> 4) & 0x3FFF) << 16;  // K-adjacent core matrices: 128 B apart
-  d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;   // 8-row groups: sbo bytes apart
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Instruction descriptor: FP32 accumulator, A/B format (kind::tf32: TF32 = 2; kind::f16: FP16 = 0,
-// BF16 = 1), K-major A and B.
-__host__ __device__ constexpr uint32_t instr_desc(uint32_t ab_format, int M, int N) {
-  return (1u << 4) | (ab_format << 7) | (ab_format << 10) | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
-}
 
 struct TcStep {
   const uint8_t* img_hi;  // nchunks x (Npad x KCB)
@@ -254,10 +93,6 @@ constexpr int STAGE_COLS = 16;             // epilogue staging: 32 rows x 16 col
 constexpr int STAGE_LD = STAGE_COLS + 1;   // its row stride (floats; odd: no bank conflicts)
 
 // Launch configurations: bytes of K per row per chunk (KCB) and operand ring depth (NS).
-// Operand formats of the tensor-core forms.
-constexpr int FMT_TF32 = 0, FMT_BF16 = 1, FMT_FP16 = 2;
-__host__ __device__ constexpr uint32_t fmt_code(int fmt) { return fmt == FMT_TF32 ? 2u : fmt == FMT_BF16 ? 1u : 0u; }
-
 template <int FMT, bool SPLIT, int KCB_, int NS>
 struct Cfg {
   static constexpr int KCB = KCB_;
@@ -1116,7 +951,6 @@ __device__ __forceinline__ void umma_f16_ts(uint32_t d, uint32_t a_tmem, uint64_
 __device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t v) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(v) : "memory");
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // 16 single columns c0 .. c0 + 15 of this warp's 32 lanes, one load each, and the wait for
 // them, in one block (so that no use of the values can be scheduled before the wait).
 __device__ __forceinline__ void tmem_ld1x16(uint32_t c0, float* v) {
@@ -1183,36 +1017,6 @@ struct TsArgs {
   uint32_t b_slot_bytes;  // bytes reserved per B part per slot
 };
 
-// 16-bit pair of a generated A value pair: FP16 or BF16, and the residual's pair for the split
-template <int FMT, bool SPLIT>
-__device__ __forceinline__ void pack_pair(float v0, float v1, uint32_t& h, uint32_t& l) {
-  if constexpr (FMT == FMT_BF16) {
-    const __nv_bfloat162 hb = __floats2bfloat162_rn(v0, v1);
-    h = *reinterpret_cast<const uint32_t*>(&hb);
-    if (SPLIT) {
-      const float2 hf = __bfloat1622float2(hb);
-      const __nv_bfloat162 lb = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
-      l = *reinterpret_cast<const uint32_t*>(&lb);
-    }
-  } else {
-    const __half2 hh = __floats2half2_rn(v0, v1);
-    h = *reinterpret_cast<const uint32_t*>(&hh);
-    if (SPLIT) {
-      const float2 hf = __half22float2(hh);
-      const __half2 lh = __floats2half2_rn(v0 - hf.x, v1 - hf.y);
-      l = *reinterpret_cast<const uint32_t*>(&lh);
-    }
-  }
-}
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // bulk copy of `bytes` from global memory to the same shared-memory offset in every CTA of the
 // cluster named by `mask`, each destination's mbarrier (same offset) receiving the bytes
 __device__ __forceinline__ void tma_load_1d_mc(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint16_t mask) {
@@ -1619,26 +1423,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
 constexpr int NSA_TSE = 2;
 constexpr int EPI_LD = 33;  // epilogue staging: 32 rows x 32 columns, row stride 33 floats
 
-// 32 consecutive TMEM columns of this warp's 32 lanes and the wait for them, in one block (no
-// use of the values can be scheduled before the wait)
-__device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 template <int FMT, bool SPLIT, int NSB>
 __global__ void __launch_bounds__(TCE_THREADS, 1) chain_tse_kernel(TsArgs a) {
   constexpr int PARTS = SPLIT ? 2 : 1;
@@ -2038,6 +1822,7 @@ std::mutex g_img_mu;
 struct TcImageCache {
   Images img[6][2];
   Images ts[6];                       // images of the TS kernel (kind::f16 forms)
+  PairImages pair[6];                 // images of the SM-pair kernel (kind::f16 forms)
   double* L[2] = {nullptr, nullptr};  // merged first two cores per side (see tc_chain_steps)
 };
 
@@ -2060,6 +1845,8 @@ void tc_cache_free(TcImageCache* c) {
     for (auto& im : f)
       if (im.buf) cudaFree(im.buf);
   for (auto& im : c->ts)
+    if (im.buf) cudaFree(im.buf);
+  for (auto& im : c->pair)
     if (im.buf) cudaFree(im.buf);
   for (double* L : c->L)
     if (L) cudaFree(L);
@@ -2223,8 +2010,9 @@ static pttk_status build_images(const pttk_tt* tt, const TcImageCache* cache, pt
   return PTTK_OK;
 }
 
-// Launch configurations. 0: the shared-memory kernel with dedicated epilogue warps and
-// double-buffered accumulators (chain_tce_kernel; the default), 128 bytes of K per chunk row;
+// Launch configurations. 0 (the default): the SM-pair kernel (chain_pair.cu) for the kind::f16 forms
+// with d >= 2 whose ranks fit it, else the shared-memory kernel with dedicated epilogue warps and
+// double-buffered accumulators (chain_tce_kernel), 128 bytes of K per chunk row;
 // 1 and 2: the shared-memory kernel without them, with {KCB, NSLOT} below; 3..5: the TS kernel
 // (A in tensor memory, a ring of 3 slots) in thread-block clusters of 1, 2 or 4 CTAs, for the
 // kind::f16 forms whose ranks fit it. A configuration whose kernel cannot hold the ranks falls
@@ -2458,10 +2246,16 @@ static pttk_status launch_tse(TsArgs a, int64_t T0, int64_t T1, size_t smem, cud
 pttk_status tc_prepare(const pttk_tt* tt, TcImageCache* cache, pttk_prec prec, int cfg, cudaStream_t s) {
   const int fi = form_index(prec);
   if (fi < 0) return set_error(PTTK_EINVAL, "not a tensor-core form");
+  const bool pair = cfg == 0 && pair_form(tt, prec);
+  if (cfg == kTcSharedA) cfg = 0;
   int KCB, NS;
   tc_config(prec, cfg, &KCB, &NS);
   Images& im = cache->img[fi][KCB == 64 ? 0 : 1];
   std::lock_guard<std::mutex> lk(g_img_mu);
+  if (pair) {
+    PairImages& pi = cache->pair[fi];
+    return pi.buf ? PTTK_OK : pair_prepare(tt, prec, pi, s);
+  }
   PTTK_TRY(ensure_merged(tt, cache));
   if ((ts_config(cfg) || tse_config(cfg)) && ts_form(prec)) {
     Images& ti = cache->ts[fi];
@@ -2503,6 +2297,9 @@ pttk_status factor_build_tc(const pttk_tt* tt, TcImageCache* cache, const float*
   if (N_s == 0 && N_t == 0) return PTTK_OK;
   PTTK_TRY(tc_prepare(tt, cache, prec, cfg, s));
   const int fi = form_index(prec);
+  if (cfg == kTcSharedA) cfg = 0;
+  else if (cfg == 0 && pair_form(tt, prec))
+    return pair_build(tt, prec, cache->pair[fi], X, N_s, Y, N_t, U, V, d_status, s);
   if (tse_config(cfg) && ts_form(prec)) {
     TsArgs a;
     size_t smem = 0;

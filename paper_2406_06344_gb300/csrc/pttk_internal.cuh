@@ -126,7 +126,9 @@ struct TcImageCache;
 TcImageCache* tc_cache_new();
 void tc_cache_free(TcImageCache* c);
 // Both factors in one persistent launch; cfg selects a launch configuration (0 = default,
-// tc_config_count() of them). Lays out the core images on first use (synchronises once).
+// tc_config_count() of them; kTcSharedA: the default's shared-memory kernel whatever the ranks).
+// Lays out the core images on first use (synchronises once).
+constexpr int kTcSharedA = 1 << 8;
 pttk_status factor_build_tc(const pttk_tt* tt, TcImageCache* cache, const float* X, int64_t N_s,
                             const float* Y, int64_t N_t, pttk_prec prec, float* U, float* V,
                             int* d_status, int cfg, cudaStream_t s);
