@@ -248,7 +248,7 @@ struct Scratch {
   template <typename T>
   pttk_status get(T** out, size_t elems) {
     void* p = nullptr;
-    const cudaError_t e = cudaMallocAsync(&p, std::max<size_t>(elems, 1) * sizeof(T), s);
+    const cudaError_t e = ws_malloc(&p, std::max<size_t>(elems, 1) * sizeof(T), s);
     if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(adjoint scratch)");
     ptrs.push_back(p);
     *out = static_cast<T*>(p);

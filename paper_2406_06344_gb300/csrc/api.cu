@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -40,6 +41,60 @@ int sm_count() {
   return count[dev];
 }
 
+namespace {
+std::mutex g_ws_mu;
+cudaMemPool_t g_ws_pool[64] = {nullptr};
+int g_ws_handles = 0;
+}  // namespace
+
+cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  int dev = 0;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone || cudaGetDevice(&dev) != cudaSuccess ||
+      dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return cudaMallocAsync(p, bytes, s);
+  }
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> lk(g_ws_mu);
+    if (!g_ws_pool[dev]) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t made = nullptr;
+      cudaError_t e = cudaMemPoolCreate(&made, &props);
+      unsigned long long keep = kWorkspaceKeep;
+      if (e == cudaSuccess) e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+      if (e != cudaSuccess) {
+        if (made) cudaMemPoolDestroy(made);
+        cudaGetLastError();
+        return cudaMallocAsync(p, bytes, s);
+      }
+      g_ws_pool[dev] = made;
+    }
+    pool = g_ws_pool[dev];
+  }
+  const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e != cudaErrorMemoryAllocation) return e;
+  // the kept workspace of finished work may be what is missing
+  cudaGetLastError();
+  cudaMemPoolTrimTo(pool, 0);
+  return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+void ws_handle_added() {
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  ++g_ws_handles;
+}
+void ws_handle_freed() {
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  if (--g_ws_handles == 0)
+    for (cudaMemPool_t pool : g_ws_pool)
+      if (pool) cudaMemPoolTrimTo(pool, 0);
+}
+
 // Target-side cores transposed to (right rank, j, left rank) so both factor chains read
 // their cores as (input rank, j, output rank).
 __global__ void orient_kernel(const double* __restrict__ G, int ra, int n, int rb,
@@ -58,6 +113,8 @@ __global__ void orient_kernel(const double* __restrict__ G, int ra, int n, int r
 
 // Handles keep their target-side oriented cores next to the cores (allocated together).
 struct pttk_tt_ext : pttk_tt {
+  pttk_tt_ext() { pttk::ws_handle_added(); }
+  ~pttk_tt_ext() { pttk::ws_handle_freed(); }
   double* tgt64 = nullptr;
   float* tgt32 = nullptr;
   pttk::TcImageCache* tc = nullptr;  // tensor-core core images, built on first use per form
@@ -226,7 +283,7 @@ pttk_status pttk_grid_entries(pttk_kernel kernel, int d, const double* src_box,
   fill_meta(&meta, kernel, d, src_box, tgt_box, d_theta, theta_box, n);
   cudaStream_t s = as_stream(stream);
   int* dstat = nullptr;
-  PTTK_CUDA(cudaMallocAsync(&dstat, sizeof(int), s));
+  PTTK_CUDA(ws_malloc(&dstat, sizeof(int), s));
   pttk_status st = PTTK_OK;
   int h = 0;
   if (cudaMemsetAsync(dstat, 0, sizeof(int), s) != cudaSuccess) st = cuda_error(cudaGetLastError(), "memset");
@@ -553,7 +610,7 @@ pttk_status pttk_apply(const void* U, const void* M, const void* V, int64_t N_s,
   cudaStream_t s = as_stream(stream);
   const bool fp64 = prec == PTTK_FP64;
   void* scratch = nullptr;
-  PTTK_CUDA(cudaMallocAsync(&scratch, apply_scratch_bytes(N_t, rs, rt, fp64), s));
+  PTTK_CUDA(ws_malloc(&scratch, apply_scratch_bytes(N_t, rs, rt, fp64), s));
   const pttk_status st = apply_run(U, M, V, N_s, N_t, rs, rt, fp64, w, out, scratch, s);
   cudaFreeAsync(scratch, s);
   return st;

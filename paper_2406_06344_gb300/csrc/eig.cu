@@ -401,10 +401,10 @@ pttk_status sym_eig_values(double* A, int k, int nb, double* d, double* e, doubl
     const int nch_max = (k + CHUNK - 1) / CHUNK;
     double *part = nullptr, *vbuf = nullptr, *wbuf = nullptr;
     unsigned* done = nullptr;
-    PTTK_CUDA(cudaMallocAsync(&part, sizeof(double) * (size_t)nb * nch_max * k, s));
-    PTTK_CUDA(cudaMallocAsync(&vbuf, sizeof(double) * (size_t)nb * k, s));
-    PTTK_CUDA(cudaMallocAsync(&wbuf, sizeof(double) * (size_t)nb * k, s));
-    PTTK_CUDA(cudaMallocAsync(&done, sizeof(unsigned) * (size_t)nb * k, s));
+    PTTK_CUDA(ws_malloc(&part, sizeof(double) * (size_t)nb * nch_max * k, s));
+    PTTK_CUDA(ws_malloc(&vbuf, sizeof(double) * (size_t)nb * k, s));
+    PTTK_CUDA(ws_malloc(&wbuf, sizeof(double) * (size_t)nb * k, s));
+    PTTK_CUDA(ws_malloc(&done, sizeof(unsigned) * (size_t)nb * k, s));
     PTTK_CUDA(cudaMemsetAsync(done, 0, sizeof(unsigned) * (size_t)nb * k, s));
     PTTK_PROF("eig_tridiag", s);
     const int gmax = std::max(1, 2 * sm_count() / nb);
@@ -472,16 +472,16 @@ pttk_status sym_eig_vectors(const double* A, const double* d, const double* e, c
   const int nclus = (int)job.size() / 2;
   int *djob = nullptr, *dz = nullptr, *dcol = nullptr;
   double *dlam = nullptr, *work = nullptr;
-  PTTK_CUDA(cudaMallocAsync(&djob, sizeof(int) * job.size(), s));
-  PTTK_CUDA(cudaMallocAsync(&dz, sizeof(int) * nsel, s));
-  PTTK_CUDA(cudaMallocAsync(&dcol, sizeof(int) * nsel, s));
-  PTTK_CUDA(cudaMallocAsync(&dlam, sizeof(double) * nsel, s));
+  PTTK_CUDA(ws_malloc(&djob, sizeof(int) * job.size(), s));
+  PTTK_CUDA(ws_malloc(&dz, sizeof(int) * nsel, s));
+  PTTK_CUDA(ws_malloc(&dcol, sizeof(int) * nsel, s));
+  PTTK_CUDA(ws_malloc(&dlam, sizeof(double) * nsel, s));
   // factors in shared memory up to k = 4900 (5 k doubles + k flags); beyond, in global memory
   const size_t ii_bytes = sizeof(double) * 5 * (size_t)k + (size_t)k;
   const int in_smem = ii_bytes <= 200 * 1024;
   if (in_smem && ii_bytes > 48 * 1024)
     PTTK_CUDA(cudaFuncSetAttribute(inverse_iteration_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ii_bytes));
-  PTTK_CUDA(cudaMallocAsync(&work, in_smem ? sizeof(double) : sizeof(double) * 6 * (size_t)k * nclus, s));
+  PTTK_CUDA(ws_malloc(&work, in_smem ? sizeof(double) : sizeof(double) * 6 * (size_t)k * nclus, s));
   PTTK_CUDA(cudaMemcpyAsync(djob, job.data(), sizeof(int) * job.size(), cudaMemcpyHostToDevice, s));
   PTTK_CUDA(cudaMemcpyAsync(dz, sel_z.data(), sizeof(int) * nsel, cudaMemcpyHostToDevice, s));
   PTTK_CUDA(cudaMemcpyAsync(dcol, sel_col.data(), sizeof(int) * nsel, cudaMemcpyHostToDevice, s));

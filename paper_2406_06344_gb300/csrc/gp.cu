@@ -226,7 +226,7 @@ pttk_status pttk_gp_kv(int kernel, int d, const double* X, int64_t N, const doub
   if (prec != PTTK_FP64 && prec != PTTK_FP32) return set_error(PTTK_EINVAL, "K v: prec must be PTTK_FP64 or PTTK_FP32");
   cudaStream_t s = as_stream(stream);
   double* part = nullptr;
-  PTTK_CUDA(cudaMallocAsync(&part, sizeof(double) * (size_t)kv_splits(N) * N, s));
+  PTTK_CUDA(ws_malloc(&part, sizeof(double) * (size_t)kv_splits(N) * N, s));
   const pttk_status st = kv_launch(kernel, d, X, N, theta[0], s2, v, out, prec == PTTK_FP32, part, s);
   cudaFreeAsync(part, s);
   return st;

@@ -427,8 +427,8 @@ pttk_status grid_coeffs_launch(int kernel, int d, int dtheta, int n, const doubl
       }
       P = std::max(P, 1);
       const size_t cnt = (size_t)n * P * KV_STRIDE;
-      PTTK_CUDA(cudaMallocAsync(&tab64, sizeof(double) * cnt, s));
-      PTTK_CUDA(cudaMallocAsync(&tab32, sizeof(float) * cnt, s));
+      PTTK_CUDA(ws_malloc(&tab64, sizeof(double) * cnt, s));
+      PTTK_CUDA(ws_malloc(&tab32, sizeof(float) * cnt, s));
       kv_table_kernel<<<n, 256, 0, s>>>(n, P, zlo, a.lo[d + 1], a.hi[d + 1], tab64, tab32); pttk::count_launch();
       PTTK_CUDA(cudaGetLastError());
       a.kv_tab = fp64 ? static_cast<const void*>(tab64) : static_cast<const void*>(tab32);

@@ -595,7 +595,7 @@ pttk_status theta_core_run(const pttk_tt* tt, const double* theta_hat, bool fp64
   for (int j = 0; j < dth; ++j) need += (size_t)tt->ranks[d + j] * tt->ranks[d + j + 1];
   need += (size_t)rs * rt * (dth > 1 ? nslices : 0);
   double* work = nullptr;
-  PTTK_CUDA(cudaMallocAsync(&work, sizeof(double) * std::max<size_t>(need, 1), s));
+  PTTK_CUDA(ws_malloc(&work, sizeof(double) * std::max<size_t>(need, 1), s));
   double* Hj[2] = {work, work + (size_t)tt->ranks[d] * tt->ranks[d + 1]};
   for (int j = 0; j < dth; ++j) {
     const int ra = tt->ranks[d + j], rb = tt->ranks[d + j + 1];
