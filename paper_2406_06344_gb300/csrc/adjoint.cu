@@ -287,8 +287,7 @@ pttk_status grad_typed(const pttk_tt* tt, const double* theta, const T* X, int64
   PTTK_TRY(theta_core_run(tt, th, true, M, s));
   PTTK_TRY(point_domain_check(tt, X, N_s, Y, N_t, fp64, tt_status_word(tt), s));
   if (prec == PTTK_FP64 || prec == PTTK_FP32) {
-    PTTK_TRY(factor_build_run(tt, true, X, N_s, prec, U, s));
-    PTTK_TRY(factor_build_run(tt, false, Y, N_t, prec, V, s));
+    PTTK_TRY(factor_build_both(tt, X, N_s, Y, N_t, prec, U, V, s));
   } else {
     // the shared-memory kernel: the theta-gradient is an FP64 result of these factors, and their last
     // FP32 bits differ between the chain kernels

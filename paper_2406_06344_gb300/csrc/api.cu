@@ -573,9 +573,7 @@ pttk_status pttk_instantiate(const pttk_tt* tt, const double* theta, const void*
   PTTK_TRY(theta_core_run(tt, th, prec == PTTK_FP64, M, s));
   PTTK_TRY(point_domain_check(tt, X, N_s, Y, N_t, prec == PTTK_FP64, tt_status_word(tt), s));
   if (prec == PTTK_FP64 || prec == PTTK_FP32) {
-    PTTK_TRY(factor_build_run(tt, true, X, N_s, prec, U, s));
-    PTTK_TRY(factor_build_run(tt, false, Y, N_t, prec, V, s));
-    return PTTK_OK;
+    return factor_build_both(tt, X, N_s, Y, N_t, prec, U, V, s);
   }
   const pttk_tt_ext* t = static_cast<const pttk_tt_ext*>(tt);
   return factor_build_tc(tt, t->tc, static_cast<const float*>(X), N_s, static_cast<const float*>(Y), N_t, prec,

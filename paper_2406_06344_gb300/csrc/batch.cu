@@ -266,9 +266,7 @@ pttk_status pttk_instantiate_batched(const pttk_batch* b, const double* thetas, 
   if (tc_form(b->prec))
     return factor_build_tc(tt, tt_tc_cache(tt), static_cast<const float*>(X), b->Ns, static_cast<const float*>(Y),
                            b->Nt, b->prec, static_cast<float*>(U), static_cast<float*>(V), status, b->cfg, s);
-  PTTK_TRY(factor_build_run(tt, true, X, b->Ns, b->prec, U, s));
-  PTTK_TRY(factor_build_run(tt, false, Y, b->Nt, b->prec, V, s));
-  return PTTK_OK;
+  return factor_build_both(tt, X, b->Ns, Y, b->Nt, b->prec, U, V, s);
 }
 
 void pttk_batch_free(pttk_batch* b) {

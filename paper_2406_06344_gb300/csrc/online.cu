@@ -138,116 +138,190 @@ __global__ void identity_rowmajor_kernel(void* M, int r, bool fp64) {
 // ---------------- factor chain (SIMT) -----------------------------------------------
 struct ChainStep {
   const void* G;  // oriented core, column-major (R_in x n x R_out)
-  int R_in, R_out, coord;
+  int R_in, R_out, coord, ct;  // ct: output columns per pass (0: the narrow form)
+  uint32_t magic;              // ceil(2^32 / R_in): k / R_in = umulhi(k, magic) (R_in > 1)
   double lo, hi;
 };
-struct ChainArgs {
+struct ChainSide {
   ChainStep st[3];
-  int nsteps, n, d, Rmax;  // Rmax: largest R (padded to 64) held in shared memory
+  const void* pts;
+  void* out;
   int64_t N;
 };
+struct ChainArgs {
+  ChainSide side[2];
+  int nsteps, n, d;
+  int64_t blocks0;  // blocks of side 0
+  int rin_max;      // largest R_in of a step
+};
 
-constexpr int CT = 64;  // output columns per tile
-constexpr int BK = 16;  // K chunk
+constexpr int BK = 16;      // values of K per chunk
+constexpr int NARROW = 16;  // steps of at most this many outputs take the narrow form
 
-// One CTA builds the factor rows of P points. Threads: (P/4) x 16, each owning a 4 x 4
-// register tile of (points, output columns).
+__device__ __forceinline__ void fma_pair(double a, const double* b, double* acc) {
+  acc[0] = fma(a, b[0], acc[0]);
+  acc[1] = fma(a, b[1], acc[1]);
+}
+__device__ __forceinline__ void fma_pair(float a, const float* b, float* acc) {
+  // the two-wide FP32 FMA: each half rounds as fmaf does
+  uint64_t x, y, z;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(x) : "f"(a));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b[0]), "f"(b[1]));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(acc[0]), "f"(acc[1]));
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(z) : "l"(x), "l"(y), "l"(z));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[0]), "=f"(acc[1]) : "l"(z));
+}
+
+// One chain step of a block's P = 16 TM points: 16 x 16 threads, each TM points x TN outputs (the pairs
+// 32 jj + 2 tx, + 1), CT = 16 TN outputs per pass. A[k][p] = T_j S_in[a] is formed chunk by chunk in
+// shared memory beside the core's chunk, which was loaded one chunk ahead into registers; the two chunk
+// buffers alternate, so a chunk costs one barrier. Every output is summed over k in order.
+template <typename T, int TM, int TN>
+__device__ void chain_step(const ChainStep& st, int n, const T* __restrict__ Bv, const T* __restrict__ Sin,
+                           T* __restrict__ Sout, T* __restrict__ As, T* __restrict__ Gs, T* __restrict__ out, int64_t p0,
+                           int64_t N, bool last) {
+  constexpr int P = 16 * TM, CT = 16 * TN, GL = CT + 4;
+  constexpr int NA = BK * P / 256, NG = BK * CT / 256;
+  const T* __restrict__ G = static_cast<const T*>(st.G);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int K = n * st.R_in;
+  for (int o0 = 0; o0 < st.R_out; o0 += CT) {
+    T acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
+    T greg[NG];
+    auto load_g = [&](int k0) {
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        const int e = tid + 256 * i, kk = e % BK, o = e / BK;
+        greg[i] = (k0 + kk < K && o0 + o < st.R_out) ? __ldg(G + (k0 + kk) + (int64_t)K * (o0 + o)) : T(0);
+      }
+    };
+    load_g(0);
+    int buf = 0;
+    for (int k0 = 0; k0 < K; k0 += BK, buf ^= 1) {
+      T* Ab = As + buf * BK * P;
+      T* Gb = Gs + buf * BK * GL;
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        const int e = tid + 256 * i;
+        Gb[(e % BK) * GL + e / BK] = greg[i];
+      }
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        const int e = tid + 256 * i, kk = e / P, p = e % P, k = k0 + kk;
+        T v = T(0);
+        if (k < K) {
+          const int j = st.R_in > 1 ? (int)__umulhi((uint32_t)k, st.magic) : k;
+          v = Bv[j * P + p] * Sin[(k - j * st.R_in) * P + p];
+        }
+        Ab[kk * P + p] = v;
+      }
+      __syncthreads();
+      if (k0 + BK < K) load_g(k0 + BK);
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) {
+        T av[TM], bv[TN];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) av[i] = Ab[kk * P + ty * TM + i];
+#pragma unroll
+        for (int j = 0; j < TN; j += 2) {
+          bv[j] = Gb[kk * GL + 16 * j + 2 * tx];
+          bv[j + 1] = Gb[kk * GL + 16 * j + 2 * tx + 1];
+        }
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; j += 2) fma_pair(av[i], bv + j, acc[i] + j);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int oc = o0 + 16 * (j & ~1) + 2 * tx + (j & 1);
+      if (oc >= st.R_out) continue;
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const int p = ty * TM + i;
+        if (last) {
+          if (p0 + p < N) out[(p0 + p) * st.R_out + oc] = acc[i][j];
+        } else {
+          Sout[oc * P + p] = acc[i][j];
+        }
+      }
+    }
+    __syncthreads();  // the chunk buffers are free again, and S_out is complete after the last pass
+  }
+}
+
+// A step of at most NARROW outputs: one output per thread at a time, the core's values read as
+// broadcasts. In the tiled form a first step (n values of K, about 10 outputs) would compute 64 columns: 10 %
+// of a d = 2 chain.
 template <typename T, int P>
-__global__ void __launch_bounds__((P / 4) * 16) chain_kernel(ChainArgs a, const T* __restrict__ pts,
-                                                             T* __restrict__ out) {
-  constexpr int NT = (P / 4) * 16;
+__device__ void chain_step_narrow(const ChainStep& st, int n, const T* __restrict__ Bv, const T* __restrict__ Sin,
+                                  T* __restrict__ Sout, T* __restrict__ out, int64_t p0, int64_t N, bool last) {
+  const T* __restrict__ G = static_cast<const T*>(st.G);
+  const int K = n * st.R_in;
+  for (int e = threadIdx.x; e < P * st.R_out; e += 256) {
+    const int p = e % P, o = e / P;
+    T acc = T(0);
+    for (int j = 0, k = 0; j < n; ++j) {
+      const T b = Bv[j * P + p];
+      for (int ar = 0; ar < st.R_in; ++ar, ++k) acc = fma(b * Sin[ar * P + p], __ldg(G + k + (int64_t)K * o), acc);
+    }
+    if (!last) Sout[o * P + p] = acc;
+    else if (p0 + p < N) out[(p0 + p) * st.R_out + o] = acc;
+  }
+  __syncthreads();
+}
+
+// Factor rows of both sides: a block takes 16 TM points of one side. TM is chosen by the point counts and
+// ranks (factor_build_run). What bounds it: FMA issue. 200k points a side, ranks 10, 63 | 63, 12, n = 20:
+// FP32 1.156 -> 0.29 ms, FP64 11.13 -> 9.9 ms (9.05 ms at the DFMA rate), against 64 points x 64 columns a
+// block, 4 x 4 a thread, one buffer and a tiled first step.
+template <typename T, int TM>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) chain_kernel(ChainArgs a) {
+  constexpr int P = 16 * TM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* Sa = reinterpret_cast<T*>(smem_raw);  // P x Rmax (point-major: Sa[p * Rmax + r])
-  T* Sb = Sa + (size_t)P * a.Rmax;
-  T* Bv = Sb + (size_t)P * a.Rmax;         // P x n basis values
-  T* As = Bv + (size_t)P * PTTK_MAX_N;     // BK x P
-  T* Gs = As + BK * P;                     // BK x CT
-
-  const int64_t p0 = (int64_t)blockIdx.x * P;
-  const int tp = threadIdx.x / 16, to = threadIdx.x % 16;
+  const int sd = (int64_t)blockIdx.x < a.blocks0 ? 0 : 1;
+  const ChainSide& side = a.side[sd];
   const int n = a.n;
-  T* Sin = Sa;
-  T* Sout = Sb;
+  T* Sin = reinterpret_cast<T*>(smem_raw);      // rin_max x P
+  T* Sout = Sin + (size_t)a.rin_max * P;
+  T* Bv = Sout + (size_t)a.rin_max * P;         // n x P basis values
+  T* As = Bv + (size_t)n * P;                   // 2 x BK x P
+  T* Gs = As + 2 * BK * P;                      // 2 x BK x (ct + 4)
+  const int64_t p0 = ((int64_t)blockIdx.x - (sd ? a.blocks0 : 0)) * P, N = side.N;
+  const T* __restrict__ pts = static_cast<const T*>(side.pts);
+  T* out = static_cast<T*>(side.out);
   // S_0 = 1 (r_0 = 1)
-  for (int p = threadIdx.x; p < P; p += NT) Sin[p * a.Rmax] = T(1);
-
+  for (int p = threadIdx.x; p < P; p += 256) Sin[p] = T(1);
   for (int si = 0; si < a.nsteps; ++si) {
-    const ChainStep st = a.st[si];
-    const T* G = static_cast<const T*>(st.G);
+    const ChainStep& st = side.st[si];
     // Chebyshev basis of this coordinate by the three-term recurrence
-    for (int p = threadIdx.x; p < P; p += NT) {
+    for (int p = threadIdx.x; p < P; p += 256) {
       const int64_t gp = p0 + p;
-      const T x = gp < a.N ? pts[gp * a.d + st.coord] : T(st.lo);
+      const T x = gp < N ? pts[gp * a.d + st.coord] : T(st.lo);
       const T xh = (T(2) * x - T(st.lo) - T(st.hi)) / (T(st.lo) - T(st.hi));
       T t0 = T(1), t1 = xh;
-      Bv[p * PTTK_MAX_N + 0] = t0;
-      if (n > 1) Bv[p * PTTK_MAX_N + 1] = t1;
+      Bv[p] = t0;
+      if (n > 1) Bv[P + p] = t1;
       for (int k = 2; k < n; ++k) {
         const T t2 = T(2) * xh * t1 - t0;
-        Bv[p * PTTK_MAX_N + k] = t2;
+        Bv[k * P + p] = t2;
         t0 = t1;
         t1 = t2;
       }
     }
     __syncthreads();
-    const int K = n * st.R_in;
-    for (int o0 = 0; o0 < st.R_out; o0 += CT) {
-      T acc[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-      for (int k0 = 0; k0 < K; k0 += BK) {
-        // A chunk: As[kk][p] = B[p, j] * S_in[p, a], k = a + R_in j
-        for (int e = threadIdx.x; e < BK * P; e += NT) {
-          const int kk = e / P, p = e % P;
-          const int k = k0 + kk;
-          T v = T(0);
-          if (k < K) {
-            const int j = k / st.R_in, ar = k % st.R_in;
-            v = Bv[p * PTTK_MAX_N + j] * Sin[p * a.Rmax + ar];
-          }
-          As[kk * P + p] = v;
-        }
-        // core chunk: Gs[kk][o] = Gs2[k, o0 + o]
-        for (int e = threadIdx.x; e < BK * CT; e += NT) {
-          const int kk = e / CT, o = e % CT;
-          const int k = k0 + kk, oc = o0 + o;
-          Gs[kk * CT + o] = (k < K && oc < st.R_out) ? G[k + (int64_t)K * oc] : T(0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-          T av[4], bv[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) av[i] = As[kk * P + tp * 4 + i];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) bv[j] = Gs[kk * CT + to * 4 + j];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-      }
-      const bool last = si == a.nsteps - 1;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int p = tp * 4 + i;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int oc = o0 + to * 4 + j;
-          if (oc >= st.R_out) continue;
-          if (last) {
-            const int64_t gp = p0 + p;
-            if (gp < a.N) out[gp * st.R_out + oc] = acc[i][j];
-          } else {
-            Sout[p * a.Rmax + oc] = acc[i][j];
-          }
-        }
-      }
+    const bool last = si == a.nsteps - 1;
+    switch (st.ct) {
+      case 0: chain_step_narrow<T, P>(st, n, Bv, Sin, Sout, out, p0, N, last); break;
+      case 64: chain_step<T, TM, 4>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
+      case 96: chain_step<T, TM, 6>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
+      default: chain_step<T, TM, 8>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
     }
-    __syncthreads();
     T* tmp = Sin;
     Sin = Sout;
     Sout = tmp;
@@ -621,59 +695,100 @@ pttk_status theta_core_run(const pttk_tt* tt, const double* theta_hat, bool fp64
   return PTTK_OK;
 }
 
-template <typename T, int P>
-static pttk_status launch_chain(const ChainArgs& a, const T* pts, T* out, cudaStream_t s) {
-  const size_t smem = sizeof(T) * ((size_t)2 * P * a.Rmax + (size_t)P * PTTK_MAX_N + BK * P + BK * CT);
-  auto kfn = chain_kernel<T, P>;
+// Oriented core pointer for a chain step (see pttk_tt::oriented).
+const void* oriented_core_ptr(const pttk_tt* tt, bool source, int k, bool fp64);
+
+template <typename T, int TM>
+static pttk_status launch_chain(ChainArgs a, int ct_max, cudaStream_t s) {
+  constexpr int P = 16 * TM;
+  const size_t smem = sizeof(T) * ((size_t)2 * P * a.rin_max + (size_t)P * a.n + 2 * BK * P + 2 * BK * (ct_max + 4));
+  auto kfn = chain_kernel<T, TM>;
   PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int64_t blocks = (a.N + P - 1) / P;
+  a.blocks0 = (a.side[0].N + P - 1) / P;
+  const int64_t blocks = a.blocks0 + (a.side[1].N + P - 1) / P;
   PTTK_PROF("chain", s);
-  kfn<<<(unsigned)blocks, (P / 4) * 16, smem, s>>>(a, pts, out); pttk::count_launch();
+  kfn<<<(unsigned)blocks, 256, smem, s>>>(a); pttk::count_launch();
   PTTK_CUDA(cudaGetLastError());
   return PTTK_OK;
 }
 
-// Oriented core pointer for a chain step (see pttk_tt::oriented).
-const void* oriented_core_ptr(const pttk_tt* tt, bool source, int k, bool fp64);
-
-pttk_status factor_build_run(const pttk_tt* tt, bool source, const void* P, int64_t N,
-                             pttk_prec prec, void* out, cudaStream_t s, int nsteps) {
-  if (N == 0) return PTTK_OK;
+// Both sides' factors (a side with N = 0 is left out) in one launch.
+static pttk_status chain_run(const pttk_tt* tt, const void* X, int64_t N_s, const void* Y, int64_t N_t, pttk_prec prec,
+                             void* U, void* V, cudaStream_t s, int nsteps) {
+  if (N_s == 0 && N_t == 0) return PTTK_OK;
   const bool fp64 = prec == PTTK_FP64;
   ChainArgs a{};
   a.nsteps = (nsteps > 0 && nsteps < tt->d) ? nsteps : tt->d;
   a.n = tt->n;
   a.d = tt->d;
-  a.N = N;
-  int rmax = 1;
-  for (int i = 0; i < a.nsteps; ++i) {
-    int rin, rout, coord;
-    const int k = oriented_core_dims(tt, source, i, &rin, &rout, &coord);
-    a.st[i].G = oriented_core_ptr(tt, source, k, fp64);
-    a.st[i].R_in = rin;
-    a.st[i].R_out = rout;
-    a.st[i].coord = coord;
-    const int bj = source ? coord : tt->d + tt->dtheta + coord;
-    a.st[i].lo = tt->box[bj][0];
-    a.st[i].hi = tt->box[bj][1];
-    rmax = std::max(rmax, std::max(rin, rout));
+  a.rin_max = 1;
+  int rmax = 1, ct_max = 0;
+  for (int sd = 0; sd < 2; ++sd) {
+    ChainSide& side = a.side[sd];
+    side.pts = sd == 0 ? X : Y;
+    side.out = sd == 0 ? U : V;
+    side.N = sd == 0 ? N_s : N_t;
+    if (side.N == 0) continue;
+    for (int i = 0; i < a.nsteps; ++i) {
+      int rin, rout, coord;
+      const int k = oriented_core_dims(tt, sd == 0, i, &rin, &rout, &coord);
+      ChainStep& st = side.st[i];
+      st.G = oriented_core_ptr(tt, sd == 0, k, fp64);
+      st.R_in = rin;
+      st.R_out = rout;
+      st.coord = coord;
+      st.magic = (uint32_t)((0x100000000ull + rin - 1) / rin);
+      // the pass width with the fewest padded columns, the widest of equals
+      st.ct = 0;
+      if (rout > NARROW) {
+        st.ct = 64;
+        for (int ct : {96, 128})
+          if ((rout + ct - 1) / ct * ct <= (rout + st.ct - 1) / st.ct * st.ct) st.ct = ct;
+      }
+      ct_max = std::max(ct_max, st.ct);
+      const int bj = sd == 0 ? coord : tt->d + tt->dtheta + coord;
+      st.lo = tt->box[bj][0];
+      st.hi = tt->box[bj][1];
+      a.rin_max = std::max(a.rin_max, rin);
+      rmax = std::max(rmax, std::max(rin, rout));
+    }
   }
-  a.Rmax = ((rmax + CT - 1) / CT) * CT;
+  // the ranks taken: 16 points' rows of the widest rank, padded to 64, twice within 200,000 bytes
   const size_t elem = fp64 ? 8 : 4;
   const size_t budget = 200000;
-  auto fits = [&](int P) {
-    return elem * ((size_t)2 * P * a.Rmax + (size_t)P * PTTK_MAX_N + BK * P + BK * CT) <= budget;
+  const size_t rpad = (size_t)(rmax + 63) / 64 * 64;
+  if (elem * (2 * 16 * rpad + 16 * PTTK_MAX_N + 16 * 16 + 16 * 64) > budget)
+    return set_error(PTTK_ENOTSUP, "TT ranks too large for the SIMT factor chain");
+  // The most points per block that shared memory holds and that still give every SM a block (a block's
+  // time hardly falls with its points, so few points want more blocks): FP32 up to 128, FP64 up to 64.
+  int tm = fp64 ? 4 : 8;
+  auto smem_of = [&](int t) {
+    const size_t P = 16 * (size_t)t;
+    return elem * (2 * P * a.rin_max + P * a.n + 2 * BK * P + 2 * BK * ((size_t)ct_max + 4));
   };
+  auto blocks_of = [&](int t) { return (N_s + 16 * t - 1) / (16 * t) + (N_t + 16 * t - 1) / (16 * t); };
+  while (tm > 1 && (smem_of(tm) > 227 * 1024 || blocks_of(tm) < sm_count())) tm /= 2;
+  if (smem_of(tm) > 227 * 1024) return set_error(PTTK_ENOTSUP, "TT ranks too large for the SIMT factor chain");
   if (fp64) {
-    if (fits(64)) return launch_chain<double, 64>(a, static_cast<const double*>(P), static_cast<double*>(out), s);
-    if (fits(32)) return launch_chain<double, 32>(a, static_cast<const double*>(P), static_cast<double*>(out), s);
-    if (fits(16)) return launch_chain<double, 16>(a, static_cast<const double*>(P), static_cast<double*>(out), s);
-  } else {
-    if (fits(64)) return launch_chain<float, 64>(a, static_cast<const float*>(P), static_cast<float*>(out), s);
-    if (fits(32)) return launch_chain<float, 32>(a, static_cast<const float*>(P), static_cast<float*>(out), s);
-    if (fits(16)) return launch_chain<float, 16>(a, static_cast<const float*>(P), static_cast<float*>(out), s);
+    if (tm == 4) return launch_chain<double, 4>(a, ct_max, s);
+    if (tm == 2) return launch_chain<double, 2>(a, ct_max, s);
+    return launch_chain<double, 1>(a, ct_max, s);
   }
-  return set_error(PTTK_ENOTSUP, "TT ranks too large for the SIMT factor chain");
+  if (tm == 8) return launch_chain<float, 8>(a, ct_max, s);
+  if (tm == 4) return launch_chain<float, 4>(a, ct_max, s);
+  if (tm == 2) return launch_chain<float, 2>(a, ct_max, s);
+  return launch_chain<float, 1>(a, ct_max, s);
+}
+
+pttk_status factor_build_run(const pttk_tt* tt, bool source, const void* P, int64_t N, pttk_prec prec, void* out,
+                             cudaStream_t s, int nsteps) {
+  return source ? chain_run(tt, P, N, nullptr, 0, prec, out, nullptr, s, nsteps)
+                : chain_run(tt, nullptr, 0, P, N, prec, nullptr, out, s, nsteps);
+}
+
+pttk_status factor_build_both(const pttk_tt* tt, const void* X, int64_t N_s, const void* Y, int64_t N_t, pttk_prec prec,
+                              void* U, void* V, cudaStream_t s) {
+  return chain_run(tt, X, N_s, Y, N_t, prec, U, V, s, 0);
 }
 
 size_t apply_scratch_bytes(int64_t N_t, int rs, int rt, bool fp64) {

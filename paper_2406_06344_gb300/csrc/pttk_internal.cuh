@@ -156,6 +156,9 @@ pttk_status theta_core_run(const pttk_tt* tt, const double* theta_hat, bool fp64
 // SIMT chain (FP64 / FP32); nsteps < d stops after that many steps (out: N x r_nsteps).
 pttk_status factor_build_run(const pttk_tt* tt, bool source, const void* P, int64_t N,
                              pttk_prec prec, void* out, cudaStream_t s, int nsteps = 0);
+// Both sides' chains in one launch.
+pttk_status factor_build_both(const pttk_tt* tt, const void* X, int64_t N_s, const void* Y, int64_t N_t,
+                              pttk_prec prec, void* U, void* V, cudaStream_t s);
 int oriented_core_dims(const pttk_tt* tt, bool source, int step, int* R_in, int* R_out, int* coord);
 // Symmetric eigendecomposition of nb k x k matrices (eig.cu): sym_eig_values tridiagonalises
 // A in place and returns all eigenvalues ascending (lam: nb x k) with d, e, tau for
