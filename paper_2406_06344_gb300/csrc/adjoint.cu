@@ -34,23 +34,76 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// partial[blk * r + c] = sum over the block's rows of A[row, c] w[row]  (A: N x r row-major)
-template <typename T>
+// A float as a double. The conversion instruction takes the FP64 pipe twice as long as an FMA here; for a
+// normal number the same bits come from four integer operations (the rare branch is volatile so that
+// the conversion is not computed ahead of it).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
+  if (e == 0 || e == 0x7f800000u) {
+    double d;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(x));
+    return d;
+  }
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// partial[(4 blk + lane) r + c] = sum over every fourth of the block's rows of A[row, c] w[row] in FP64
+// (A: N x r row-major). Threads are 4 row lanes x 64 column groups of VW consecutive columns (VW = 4
+// when the rows are 16-byte aligned, else 1), four rows of loads in flight each.
+template <typename T, int VW>
 __global__ void __launch_bounds__(256) weighted_colsum(const T* __restrict__ A, const T* __restrict__ w,
                                                        int64_t N, int r, double* __restrict__ partial) {
   const int64_t per = (N + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = std::min<int64_t>(N, r0 + per);
-  for (int c = threadIdx.x; c < r; c += blockDim.x) {
-    double acc = 0.0;
-    for (int64_t i = r0; i < r1; ++i) acc = fma((double)A[i * r + c], (double)w[i], acc);
-    partial[(int64_t)blockIdx.x * r + c] = acc;
+  const int cl = threadIdx.x & 63, rl = threadIdx.x >> 6;
+  for (int c = cl * VW; c < r; c += 64 * VW) {  // with VW = 4, r is a multiple of 4
+    double acc[VW];
+#pragma unroll
+    for (int q = 0; q < VW; ++q) acc[q] = 0.0;
+    int64_t i = r0 + rl;
+    for (; i + 12 < r1; i += 16) {
+      T v[4][VW];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const T* src = A + (i + 4 * u) * r + c;
+        if constexpr (VW == 4 && sizeof(T) == 4) {
+          const float4 x = *reinterpret_cast<const float4*>(src);
+          v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+        } else {
+#pragma unroll
+          for (int q = 0; q < VW; ++q) v[u][q] = src[q];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const double wr = widen(w[i + 4 * u]);
+#pragma unroll
+        for (int q = 0; q < VW; ++q) acc[q] = fma(widen(v[u][q]), wr, acc[q]);
+      }
+    }
+    for (; i < r1; i += 4) {
+      const double wr = widen(w[i]);
+#pragma unroll
+      for (int q = 0; q < VW; ++q) acc[q] = fma(widen(A[i * r + c + q]), wr, acc[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < VW; ++q) partial[(4 * (int64_t)blockIdx.x + rl) * r + c + q] = acc[q];
   }
 }
 
-__global__ void sum_partials(const double* __restrict__ partial, int nparts, int r, double* __restrict__ out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < r; c += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int b = 0; b < nparts; ++b) acc += partial[(int64_t)b * r + c];
+// out[c] = sum over the partial rows, one block per column, in a fixed order
+__global__ void __launch_bounds__(256) sum_partials(const double* __restrict__ partial, int nparts, int r,
+                                                    double* __restrict__ out) {
+  __shared__ double red[8];
+  const int c = blockIdx.x;
+  double acc = 0.0;
+  for (int b = threadIdx.x; b < nparts; b += 256) acc += partial[(int64_t)b * r + c];
+  acc = warp_sum_d(acc);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) acc += red[k];
     out[c] = acc;
   }
 }
@@ -73,53 +126,92 @@ __device__ void cheb_row(double x, int n, bool deriv, double scale, double* t) {
   }
 }
 
-// Contraction of a theta core G (ra x n x rb, column-major) with the Chebyshev (or derivative)
-// vector of th, applied to a vector on one side:
+// Contractions of theta cores G (ra x n x rb, column-major) with the Chebyshev (or derivative) vector of
+// th, applied to a vector on one side, up to four in one launch (blockIdx.y), one block per output:
 //   left  (side 0): out[c] = sum_{a,k} x[a] G[a, k, c] t[k]      (x: ra, out: rb)
 //   right (side 1): out[a] = sum_{k,c} G[a, k, c] t[k] x[c]      (x: rb, out: ra)
-__global__ void core_vec(const double* __restrict__ G, int ra, int n, int rb, double th, bool deriv,
-                        double scale, const double* __restrict__ x, int side, double* __restrict__ out) {
-  double t[PTTK_MAX_N];
-  cheb_row(th, n, deriv, scale, t);
-  const int m = side == 0 ? rb : ra;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= m) return;
+// A block's 256 threads keep their loads in flight together: what bounds it is their latency.
+struct CoreVec {
+  const double* G;
+  const double* x;
+  double* out;
+  double th, scale;
+  int ra, rb, side, deriv;
+};
+struct CoreVecs {
+  CoreVec t[4];
+};
+__global__ void __launch_bounds__(256) core_vecs(CoreVecs v, int n) {
+  const CoreVec c = v.t[blockIdx.y];
+  const int o = blockIdx.x;
+  if (o >= (c.side == 0 ? c.rb : c.ra)) return;
+  __shared__ double t[PTTK_MAX_N];
+  __shared__ double red[8];
+  if (threadIdx.x == 0) {
+    double tl[PTTK_MAX_N];
+    cheb_row(c.th, n, c.deriv != 0, c.scale, tl);
+    for (int k = 0; k < n; ++k) t[k] = tl[k];
+  }
+  __syncthreads();
   double acc = 0.0;
-  if (side == 0) {
-    const int c = warp;
-    for (int64_t e = lane; e < (int64_t)ra * n; e += 32) {
-      const int a = (int)(e % ra), k = (int)(e / ra);
-      acc = fma(x[a] * t[k], G[a + (int64_t)ra * (k + (int64_t)n * c)], acc);
+  if (c.side == 0) {
+    const double* g = c.G + (int64_t)c.ra * n * o;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < c.ra * n; e += 256) {
+      const int k = e / c.ra;
+      acc = fma(c.x[e - k * c.ra] * t[k], g[e], acc);
     }
   } else {
-    const int a = warp;
-    for (int64_t e = lane; e < (int64_t)n * rb; e += 32) {
-      const int k = (int)(e % n), c = (int)(e / n);
-      acc = fma(t[k] * x[c], G[a + (int64_t)ra * (k + (int64_t)n * c)], acc);
+    const double* g = c.G + o;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n * c.rb; e += 256) {
+      const int q = e / n;
+      acc = fma(t[e - q * n] * c.x[q], g[(int64_t)c.ra * e], acc);
     }
   }
   acc = warp_sum_d(acc);
-  if (lane == 0) out[warp] = acc;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) acc += red[i];
+    c.out[o] = acc;
+  }
 }
 
-// out[i] = sum_j M[i, j] x[j] (M row-major m x k, FP64), one warp per row; or a dot product
-__global__ void matvec_rows(const double* __restrict__ M, int m, int k, const double* __restrict__ x,
-                            double* __restrict__ out) {
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (row >= m) return;
+// out[i] = x_i . y_i (r_i values), up to three dot products, one block each
+struct Dots {
+  const double *x[3], *y[3];
+  int r[3];
+};
+__global__ void __launch_bounds__(256) dots(Dots d, double* __restrict__ out) {
+  __shared__ double red[8];
+  const int i = blockIdx.x;
   double acc = 0.0;
-  for (int j = lane; j < k; j += 32) acc = fma(M[(int64_t)row * k + j], x[j], acc);
+  for (int k = threadIdx.x; k < d.r[i]; k += 256) acc = fma(d.x[i][k], d.y[i][k], acc);
   acc = warp_sum_d(acc);
-  if (lane == 0) out[row] = acc;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) acc += red[k];
+    out[i] = acc;
+  }
 }
 
-// q[k] = sum_o Gs[k + K o] g[o]  (oriented core K x R_out, column-major)
+// q[k] = sum_o Gs[k + K o] g[o]  (oriented core K x R_out, column-major): 32 values of k a block, the
+// warps taking every eighth o, added in a fixed order
 template <typename T>
-__global__ void core_times_vec(const T* __restrict__ Gs, int K, int R, const double* __restrict__ g,
-                               T* __restrict__ q) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int o = 0; o < R; ++o) acc = fma((double)Gs[k + (int64_t)K * o], g[o], acc);
+__global__ void __launch_bounds__(256) core_times_vec(const T* __restrict__ Gs, int K, int R, const double* __restrict__ g,
+                                                      T* __restrict__ q) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int k = blockIdx.x * 32 + lane;
+  double acc = 0.0;
+  if (k < K)
+    for (int o = w; o < R; o += 8) acc = fma((double)Gs[k + (int64_t)K * o], g[o], acc);
+  red[w][lane] = acc;
+  __syncthreads();
+  if (w == 0 && k < K) {
+    for (int i = 1; i < 8; ++i) acc += red[i][lane];
     q[k] = (T)acc;
   }
 }
@@ -222,8 +314,210 @@ __global__ void __launch_bounds__(256) chain_back_step(const T* __restrict__ X, 
   }
 }
 
-unsigned nblk(int64_t work, int per = 256) {
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + per - 1) / per, (int64_t)sm_count() * 8));
+// ---------------- reverse pass in one kernel ----------------------------------------------------
+// dL/dX of the source points, one thread per point, nothing per point in memory but X, w and dX.
+// With q[b + R_2 j] = (G_d^{2} g)[b, j] and w_p:
+//   S_1 = B_1 G_1, S_2[b] = sum_{a,j} S_1[a] T_j(x_2) G_2[a, j, b]               (forward again)
+//   e_j = sum_b S_2[b] q[b, j],  dL/dx_3 = w sum_j T_j'(x_3) e_j,  gbar_2[b] = w sum_j T_j(x_3) q[b, j]
+//   Q[a, j] = sum_b gbar_2[b] G_2[a, j, b],  dL/dx_2 = sum_{a,j} S_1[a] T_j'(x_2) Q[a, j],
+//   gbar_1[a] = sum_j T_j(x_2) Q[a, j],  dL/dx_1 = sum_{a,j} gbar_1[a] G_1[j, a] T_j'(x_1)
+// (d = 2 lacks the middle step, d = 1 has the last alone.) The rows G_2[a, j, :] sit in shared memory,
+// read as broadcasts; S_2 and gbar_2 (RB values, R_2 padded) in registers; the scalars that the loops
+// index (T_j(x_2), T_j'(x_2), S_1, gbar_1) in shared memory, one column per thread. About
+// 11k FMAs a point at ranks 9, 44: at N = 500k, n = 12 the separate kernels (S_1, S_2, Q and gbar
+// in memory, shared-memory atomics per term) took 16.4 ms.
+// The bases are formed in FP64 and rounded to T.
+constexpr int AF_THREADS = 128;
+
+struct AdjArgs {
+  int d, n, r1, r2;
+  double lo[3], hi[3];
+  int coord[3];
+  const void* g1;  // oriented cores, column-major (R_in x n x R_out)
+  const void* g2;
+  const void* q;   // (R_in of the last step) x n, column-major
+};
+
+// T_j(x) and T_j'(x) dxhat/dx = j U_{j-1}(x) dxhat/dx, j < n, handed to f(j, t, dt)
+template <typename F>
+__device__ __forceinline__ void cheb_each(double x, double lo, double hi, int n, F&& f) {
+  const double xh = (2.0 * x - lo - hi) / (lo - hi), sc = 2.0 / (lo - hi), x2 = 2.0 * xh;
+  double t0 = 1.0, t1 = xh, u0 = 0.0, u1 = sc, k = 1.0;
+  f(0, 1.0, 0.0);
+  for (int j = 1; j < n; ++j) {
+    f(j, t1, k * u1);
+    const double t2 = fma(x2, t1, -t0), u2 = fma(x2, u1, -u0);
+    t0 = t1;
+    t1 = t2;
+    u0 = u1;
+    u1 = u2;
+    k += 1.0;
+  }
+}
+
+template <typename T>
+size_t adj_smem(int d, int n, int r1, int rb) {
+  // G_1 (n x r1), q (n x rlast), G_2 (r1 n x rb), then per thread T_1', T_2, T_2' (n each), S_1, gbar_1 (r1 each)
+  const size_t shared = (size_t)n * r1 + (size_t)n * (d == 3 ? rb : d == 2 ? r1 : 1) + (d == 3 ? (size_t)r1 * n * rb : 0);
+  const size_t per = (size_t)3 * n + 2 * r1;
+  return sizeof(T) * ((shared + 3) / 4 * 4 + per * AF_THREADS);
+}
+
+template <typename T, int D, int RB>
+__global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, const T* __restrict__ X, int64_t N,
+                                                                 const T* __restrict__ w, T* __restrict__ dX) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = a.n, r1 = a.r1, tid = threadIdx.x;
+  // rows of the last step's input: S_2 (d = 3, padded), S_1 (d = 2), 1 (d = 1)
+  const int rl = D == 3 ? RB : D == 2 ? r1 : 1;
+  T* G2 = reinterpret_cast<T*>(smem_raw);                 // [a][j][RB]
+  T* q = G2 + (D == 3 ? (size_t)r1 * n * RB : 0);         // [j][rl]
+  T* G1 = q + (size_t)n * rl;                             // [a][j]
+  const size_t shared = (size_t)n * r1 + (size_t)n * rl + (D == 3 ? (size_t)r1 * n * RB : 0);
+  T* priv = reinterpret_cast<T*>(smem_raw) + (shared + 3) / 4 * 4 + tid;
+  T* T2 = priv;                          // [j] at stride AF_THREADS
+  T* D2 = T2 + n * AF_THREADS;
+  T* D1 = D2 + n * AF_THREADS;
+  T* S1 = D1 + n * AF_THREADS;
+  T* B1 = S1 + r1 * AF_THREADS;
+  const int rlast = D == 3 ? a.r2 : D == 2 ? r1 : 1;
+  if (D == 3)
+    for (int e = tid; e < r1 * n * RB; e += AF_THREADS) {
+      const int b = e % RB, aj = e / RB, j = aj % n, al = aj / n;
+      G2[e] = b < a.r2 ? static_cast<const T*>(a.g2)[al + (size_t)r1 * (j + (size_t)n * b)] : T(0);
+    }
+  for (int e = tid; e < n * rl; e += AF_THREADS) {
+    const int b = e % rl, j = e / rl;
+    q[e] = b < rlast ? static_cast<const T*>(a.q)[b + (size_t)rlast * j] : T(0);
+  }
+  if (D >= 2)
+    for (int e = tid; e < n * r1; e += AF_THREADS) {
+      const int j = e % n, al = e / n;
+      G1[e] = static_cast<const T*>(a.g1)[j + (size_t)n * al];
+    }
+  __syncthreads();
+  for (int64_t p = (int64_t)blockIdx.x * AF_THREADS + tid; p < N; p += (int64_t)gridDim.x * AF_THREADS) {
+    const T wp = w[p];
+    double x[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) x[i] = (double)X[p * D + a.coord[i]];
+    if constexpr (D == 1) {
+      T acc = T(0);
+      cheb_each(x[0], a.lo[0], a.hi[0], n, [&](int j, double, double dt) { acc = fma((T)dt, q[j], acc); });
+      dX[p] = acc * wp;
+    } else {
+      // S_1
+      for (int al = 0; al < r1; ++al) S1[al * AF_THREADS] = T(0);
+      cheb_each(x[0], a.lo[0], a.hi[0], n, [&](int j, double t, double dt) {
+        const T tj = (T)t;
+        D1[j * AF_THREADS] = (T)dt;
+        for (int al = 0; al < r1; ++al) S1[al * AF_THREADS] = fma(tj, G1[al * n + j], S1[al * AF_THREADS]);
+      });
+      if constexpr (D == 3) {
+        cheb_each(x[1], a.lo[1], a.hi[1], n, [&](int j, double t, double dt) {
+          T2[j * AF_THREADS] = (T)t;
+          D2[j * AF_THREADS] = (T)dt;
+        });
+        T s2[RB], gb[RB];
+#pragma unroll
+        for (int b = 0; b < RB; ++b) s2[b] = gb[b] = T(0);
+        for (int al = 0; al < r1; ++al) {
+          const T sa = S1[al * AF_THREADS];
+          const T* row = G2 + (size_t)al * n * RB;
+          for (int j = 0; j < n; ++j, row += RB) {
+            const T m = sa * T2[j * AF_THREADS];
+#pragma unroll
+            for (int b = 0; b < RB; ++b) s2[b] = fma(m, row[b], s2[b]);
+          }
+        }
+        T dx3 = T(0);
+        cheb_each(x[2], a.lo[2], a.hi[2], n, [&](int j, double t, double dt) {
+          const T tj = (T)t * wp;
+          const T* row = q + j * RB;
+          T e[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+          for (int b = 0; b < RB; ++b) {
+            gb[b] = fma(tj, row[b], gb[b]);
+            e[b & 3] = fma(s2[b], row[b], e[b & 3]);
+          }
+          dx3 = fma((T)dt, (e[0] + e[1]) + (e[2] + e[3]), dx3);
+        });
+        T dx2 = T(0);
+        for (int al = 0; al < r1; ++al) {
+          const T sa = S1[al * AF_THREADS];
+          const T* row = G2 + (size_t)al * n * RB;
+          T g1a = T(0), da = T(0);
+          for (int j = 0; j < n; ++j, row += RB) {
+            T e[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+            for (int b = 0; b < RB; ++b) e[b & 3] = fma(gb[b], row[b], e[b & 3]);
+            const T qv = (e[0] + e[1]) + (e[2] + e[3]);
+            da = fma(D2[j * AF_THREADS], qv, da);
+            g1a = fma(T2[j * AF_THREADS], qv, g1a);
+          }
+          dx2 = fma(sa, da, dx2);
+          B1[al * AF_THREADS] = g1a;
+        }
+        dX[p * D + a.coord[2]] = dx3 * wp;
+        dX[p * D + a.coord[1]] = dx2;
+      } else {
+        for (int al = 0; al < r1; ++al) B1[al * AF_THREADS] = T(0);
+        T dx2 = T(0);
+        cheb_each(x[1], a.lo[1], a.hi[1], n, [&](int j, double t, double dt) {
+          const T tj = (T)t * wp;
+          const T* row = q + j * r1;
+          T e = T(0);
+          for (int al = 0; al < r1; ++al) {
+            B1[al * AF_THREADS] = fma(tj, row[al], B1[al * AF_THREADS]);
+            e = fma(S1[al * AF_THREADS], row[al], e);
+          }
+          dx2 = fma((T)dt, e, dx2);
+        });
+        dX[p * D + a.coord[1]] = dx2 * wp;
+      }
+      T dx1 = T(0);
+      for (int j = 0; j < n; ++j) {
+        T e = T(0);
+        for (int al = 0; al < r1; ++al) e = fma(B1[al * AF_THREADS], G1[al * n + j], e);
+        dx1 = fma(D1[j * AF_THREADS], e, dx1);
+      }
+      dX[p * D + a.coord[0]] = dx1;
+    }
+  }
+}
+
+template <typename T, int D, int RB>
+pttk_status launch_adj(const AdjArgs& a, const T* X, int64_t N, const T* w, T* dX, cudaStream_t s) {
+  auto kfn = adj_reverse_kernel<T, D, RB>;
+  const size_t smem = adj_smem<T>(D, a.n, a.r1, RB);
+  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 1;
+  PTTK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, AF_THREADS, smem));
+  const int64_t blocks = std::min<int64_t>((N + AF_THREADS - 1) / AF_THREADS, (int64_t)sm_count() * std::max(per_sm, 1));
+  kfn<<<(unsigned)blocks, AF_THREADS, smem, s>>>(a, X, N, w, dX);
+  pttk::count_launch();
+  PTTK_CUDA(cudaGetLastError());
+  return PTTK_OK;
+}
+
+// Padded R_2 of the one-kernel reverse pass; 0 where its registers (R_2 <= 64) or shared memory do not
+// hold the ranks (the separate kernels then take the call).
+template <typename T>
+int adj_fused_rb(int d, int n, int r1, int r2) {
+  const int rb = d < 3 ? 16 : r2 <= 16 ? 16 : r2 <= 32 ? 32 : r2 <= 48 ? 48 : r2 <= 64 ? 64 : 0;
+  return rb && adj_smem<T>(d, n, r1, rb) <= 220 * 1024 ? rb : 0;
+}
+
+template <typename T>
+pttk_status adj_reverse(int rb, const AdjArgs& a, const T* X, int64_t N, const T* w, T* dX, cudaStream_t s) {
+  if (a.d == 1) return launch_adj<T, 1, 16>(a, X, N, w, dX, s);
+  if (a.d == 2) return launch_adj<T, 2, 16>(a, X, N, w, dX, s);
+  switch (rb) {
+    case 16: return launch_adj<T, 3, 16>(a, X, N, w, dX, s);
+    case 32: return launch_adj<T, 3, 32>(a, X, N, w, dX, s);
+    case 48: return launch_adj<T, 3, 48>(a, X, N, w, dX, s);
+    default: return launch_adj<T, 3, 64>(a, X, N, w, dX, s);
+  }
 }
 
 template <typename T>
@@ -233,8 +527,10 @@ pttk_status weighted_sum(const T* A, const T* w, int64_t N, int r, double* out, 
     PTTK_CUDA(cudaMemsetAsync(out, 0, sizeof(double) * r, s));
     return PTTK_OK;
   }
-  weighted_colsum<T><<<nparts, 256, 0, s>>>(A, w, N, r, partial); pttk::count_launch();
-  sum_partials<<<nblk(r), 256, 0, s>>>(partial, nparts, r, out); pttk::count_launch();
+  if (r % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0) weighted_colsum<T, 4><<<nparts, 256, 0, s>>>(A, w, N, r, partial);
+  else weighted_colsum<T, 1><<<nparts, 256, 0, s>>>(A, w, N, r, partial);
+  pttk::count_launch();
+  sum_partials<<<r, 256, 0, s>>>(partial, 4 * nparts, r, out); pttk::count_launch();
   PTTK_CUDA(cudaGetLastError());
   return PTTK_OK;
 }
@@ -249,7 +545,7 @@ struct Scratch {
   pttk_status get(T** out, size_t elems) {
     void* p = nullptr;
     const cudaError_t e = ws_malloc(&p, std::max<size_t>(elems, 1) * sizeof(T), s);
-    if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(adjoint scratch)");
+    if (e != cudaSuccess) return cuda_error(e, "adjoint scratch");
     ptrs.push_back(p);
     *out = static_cast<T*>(p);
     return PTTK_OK;
@@ -265,12 +561,11 @@ pttk_status grad_typed(const pttk_tt* tt, const double* theta, const T* X, int64
   const bool fp64 = sizeof(T) == 8;
   Scratch sc{{}, s};
   T *U, *V;
-  double *M, *a, *b, *g, *partial, *small;
+  double *a, *b, *g, *partial, *small;
   PTTK_TRY(sc.get(&U, (size_t)N_s * rs));
   PTTK_TRY(sc.get(&V, (size_t)N_t * rt));
-  PTTK_TRY(sc.get(&M, (size_t)rs * rt));
-  const int nparts = (int)std::max<int64_t>(1, std::min<int64_t>((std::max(N_s, N_t) + 1023) / 1024, sm_count() * 4));
-  PTTK_TRY(sc.get(&partial, (size_t)nparts * std::max(rs, rt)));
+  const int nparts = (int)std::max<int64_t>(1, std::min<int64_t>((std::max(N_s, N_t) + 255) / 256, sm_count() * 4));
+  PTTK_TRY(sc.get(&partial, (size_t)4 * nparts * std::max(rs, rt)));
   PTTK_TRY(sc.get(&a, rs));
   PTTK_TRY(sc.get(&b, rt));
   PTTK_TRY(sc.get(&g, rs));
@@ -278,13 +573,12 @@ pttk_status grad_typed(const pttk_tt* tt, const double* theta, const T* X, int64
   for (int k = 0; k <= D; ++k) rmax = std::max(rmax, tt->ranks[k]);
   PTTK_TRY(sc.get(&small, (size_t)8 * rmax + 8));
 
-  // forward: H (FP64), U, V in the requested form
+  // forward: U, V in the requested form
   double th[PTTK_MAX_D];
   for (int j = 0; j < dth; ++j) {
     const double lo = tt->box[d + j][0], hi = tt->box[d + j][1];
     th[j] = (2.0 * theta[j] - lo - hi) / (lo - hi);
   }
-  PTTK_TRY(theta_core_run(tt, th, true, M, s));
   PTTK_TRY(point_domain_check(tt, X, N_s, Y, N_t, fp64, tt_status_word(tt), s));
   if (prec == PTTK_FP64 || prec == PTTK_FP32) {
     PTTK_TRY(factor_build_both(tt, X, N_s, Y, N_t, prec, U, V, s));
@@ -297,76 +591,96 @@ pttk_status grad_typed(const pttk_tt* tt, const double* theta, const T* X, int64
   }
   PTTK_TRY(weighted_sum<T>(U, w, N_s, rs, a, partial, nparts, s));
   PTTK_TRY(weighted_sum<T>(V, z, N_t, rt, b, partial, nparts, s));
-  matvec_rows<<<(unsigned)(((int64_t)rs * 32 + 255) / 256), 256, 0, s>>>(M, rs, rt, b, g); pttk::count_launch();  // g = H b
-  double* Lbuf = small;
-  matvec_rows<<<1, 32, 0, s>>>(a, 1, rs, g, Lbuf); pttk::count_launch();  // L = a . g
-
-  // dL/dtheta
-  if (dtheta && dth > 0) {
-    double* dth_dev = small + 1;
-    double* u = small + 8;          // rmax
-    double* v = u + rmax;           // rmax
-    double* u2 = v + rmax;          // rmax
-    double* v2 = u2 + rmax;         // rmax
+  // g = H b, L = a^T H b and dL/dtheta_j through vectors only: with one parameter g = H_1 b, L = a . g,
+  // u = H_1'^T a, dtheta = u . b; with two v = H_2 b, v' = H_2' b, u = H_1^T a, u' = H_1'^T a, g = H_1 v,
+  // L = u . v, dtheta = (u' . v, u . v').
+  double *u = small + 8, *u1 = u + rmax, *v = u1 + rmax, *v1 = v + rmax;
+  Dots dt{};
+  int ndots = 1;
+  if (dth == 0) {
+    PTTK_CUDA(cudaMemcpyAsync(g, b, sizeof(double) * rs, cudaMemcpyDeviceToDevice, s));
+    dt = Dots{{a}, {g}, {rs}};
+  } else {
     const double* G1 = tt->cores64 + tt->core_off[d];
-    const int r0 = tt->ranks[d], r1 = tt->ranks[d + 1];
+    const int r0 = tt->ranks[d], r1 = tt->ranks[d + 1], r2 = dth == 2 ? tt->ranks[d + 2] : 0;
     const double sc1 = 2.0 / (tt->box[d][0] - tt->box[d][1]);
+    auto grid = [&](int count) { return dim3((unsigned)rmax, (unsigned)count); };
     if (dth == 1) {
-      // a^T H1' b: u = H1'^T a (r1), then u . b
-      core_vec<<<(unsigned)((r1 * 32 + 255) / 256), 256, 0, s>>>(G1, r0, n, r1, th[0], true, sc1, a, 0, u); pttk::count_launch();
-      matvec_rows<<<1, 32, 0, s>>>(u, 1, r1, b, dth_dev); pttk::count_launch();
+      CoreVecs cv{{{G1, b, g, th[0], 1.0, r0, r1, 1, 0}, {G1, a, u1, th[0], sc1, r0, r1, 0, 1}}};
+      core_vecs<<<grid(2), 256, 0, s>>>(cv, n); pttk::count_launch();
+      dt = Dots{{a, u1}, {g, b}, {r0, r1}};
+      ndots = 2;
     } else {
       const double* G2 = tt->cores64 + tt->core_off[d + 1];
-      const int r2 = tt->ranks[d + 2];
       const double sc2 = 2.0 / (tt->box[d + 1][0] - tt->box[d + 1][1]);
-      // u = H1'^T a, v = H2 b, u2 = H1^T a, v2 = H2' b; dtheta = (u . v, u2 . v2)
-      { core_vec<<<(unsigned)((r1 * 32 + 255) / 256), 256, 0, s>>>(G1, r0, n, r1, th[0], true, sc1, a, 0, u); pttk::count_launch(); }
-      core_vec<<<(unsigned)((r1 * 32 + 255) / 256), 256, 0, s>>>(G2, r1, n, r2, th[1], false, 1.0, b, 1, v); pttk::count_launch();
-      core_vec<<<(unsigned)((r1 * 32 + 255) / 256), 256, 0, s>>>(G1, r0, n, r1, th[0], false, 1.0, a, 0, u2); pttk::count_launch();
-      core_vec<<<(unsigned)((r1 * 32 + 255) / 256), 256, 0, s>>>(G2, r1, n, r2, th[1], true, sc2, b, 1, v2); pttk::count_launch();
-      matvec_rows<<<1, 32, 0, s>>>(u, 1, r1, v, dth_dev); pttk::count_launch();
-      matvec_rows<<<1, 32, 0, s>>>(u2, 1, r1, v2, dth_dev + 1); pttk::count_launch();
+      CoreVecs cv{{{G2, b, v, th[1], 1.0, r1, r2, 1, 0}, {G2, b, v1, th[1], sc2, r1, r2, 1, 1},
+                   {G1, a, u, th[0], 1.0, r0, r1, 0, 0}, {G1, a, u1, th[0], sc1, r0, r1, 0, 1}}};
+      core_vecs<<<grid(4), 256, 0, s>>>(cv, n); pttk::count_launch();
+      CoreVecs cg{{{G1, v, g, th[0], 1.0, r0, r1, 1, 0}}};
+      core_vecs<<<grid(1), 256, 0, s>>>(cg, n); pttk::count_launch();
+      dt = Dots{{u, u1, u}, {v, v, v1}, {r1, r1, r1}};
+      ndots = 3;
     }
   }
+  dots<<<ndots, 256, 0, s>>>(dt, small); pttk::count_launch();
 
   // dL/dX by the reverse pass (SIMT, in the precision of X)
   if (dX && N_s > 0) {
     PTTK_PROF("adjoint", s);
-    const pttk_prec simt = fp64 ? PTTK_FP64 : PTTK_FP32;
-    std::vector<T*> Sbuf(d, nullptr);  // Sbuf[i] = S_i (N x r_i), i = 1..d-1
-    for (int i = 1; i < d; ++i) {
-      PTTK_TRY(sc.get(&Sbuf[i], (size_t)N_s * tt->ranks[i]));
-      PTTK_TRY(factor_build_run(tt, true, X, N_s, simt, Sbuf[i], s, i));
-    }
     // last step: rank-one adjoint w_p g
     int rin, rout, coord;
     oriented_core_dims(tt, true, d - 1, &rin, &rout, &coord);
     const T* Gs_last = static_cast<const T*>(oriented_core_ptr(tt, true, d - 1, fp64));
     T* q;
     PTTK_TRY(sc.get(&q, (size_t)n * rin));
-    core_times_vec<T><<<nblk((int64_t)n * rin), 256, 0, s>>>(Gs_last, n * rin, rout, g, q); pttk::count_launch();
-    T *gbar = nullptr, *gnext = nullptr, *Q = nullptr;
-    size_t qmax = 0;
-    for (int i = 0; i < d - 1; ++i) qmax = std::max<size_t>(qmax, (size_t)n * tt->ranks[i]);
-    if (d > 1) {
-      PTTK_TRY(sc.get(&gbar, (size_t)N_s * rmax));
-      PTTK_TRY(sc.get(&gnext, (size_t)N_s * rmax));
-      PTTK_TRY(sc.get(&Q, (size_t)N_s * qmax));
-    }
-    for (int i = d - 1; i >= 0; --i) {
-      oriented_core_dims(tt, true, i, &rin, &rout, &coord);
-      const double lo = tt->box[coord][0], hi = tt->box[coord][1];
-      const int K = n * rin;
-      if (i < d - 1) {
-        const T* Gs = static_cast<const T*>(oriented_core_ptr(tt, true, i, fp64));
-        dim3 grid((unsigned)((K + 63) / 64), (unsigned)((N_s + 63) / 64));
-        gemm_gbar_core<T><<<grid, 256, 0, s>>>(gbar, Gs, N_s, rout, K, Q); pttk::count_launch();
+    core_times_vec<T><<<(unsigned)((n * rin + 31) / 32), 256, 0, s>>>(Gs_last, n * rin, rout, g, q); pttk::count_launch();
+    const int rb = adj_fused_rb<T>(d, n, d > 1 ? tt->ranks[1] : 1, d > 2 ? tt->ranks[2] : 1);
+    if (rb) {
+      AdjArgs ar{};
+      ar.d = d;
+      ar.n = n;
+      ar.r1 = d > 1 ? tt->ranks[1] : 1;
+      ar.r2 = d > 2 ? tt->ranks[2] : 1;
+      for (int i = 0; i < d; ++i) {
+        int ri, ro;
+        oriented_core_dims(tt, true, i, &ri, &ro, &ar.coord[i]);
+        ar.lo[i] = tt->box[ar.coord[i]][0];
+        ar.hi[i] = tt->box[ar.coord[i]][1];
       }
-      const size_t smem = sizeof(T) * 8 * (PTTK_MAX_N + rin);
-      chain_back_step<T><<<(unsigned)((N_s + 7) / 8), 256, smem, s>>>(
-          X, d, coord, lo, hi, n, N_s, rin, i > 0 ? Sbuf[i] : nullptr, i < d - 1 ? Q : nullptr, w,
-          i == d - 1 ? q : nullptr, i > 0 ? gnext : nullptr, dX); pttk::count_launch();
-      std::swap(gbar, gnext);
+      ar.g1 = oriented_core_ptr(tt, true, 0, fp64);
+      ar.g2 = d > 2 ? oriented_core_ptr(tt, true, 1, fp64) : nullptr;
+      ar.q = q;
+      PTTK_TRY(adj_reverse<T>(rb, ar, X, N_s, w, dX, s));
+    } else {
+      const pttk_prec simt = fp64 ? PTTK_FP64 : PTTK_FP32;
+      std::vector<T*> Sbuf(d, nullptr);  // Sbuf[i] = S_i (N x r_i), i = 1..d-1
+      for (int i = 1; i < d; ++i) {
+        PTTK_TRY(sc.get(&Sbuf[i], (size_t)N_s * tt->ranks[i]));
+        PTTK_TRY(factor_build_run(tt, true, X, N_s, simt, Sbuf[i], s, i));
+      }
+      T *gbar = nullptr, *gnext = nullptr, *Q = nullptr;
+      size_t qmax = 0;
+      for (int i = 0; i < d - 1; ++i) qmax = std::max<size_t>(qmax, (size_t)n * tt->ranks[i]);
+      if (d > 1) {
+        PTTK_TRY(sc.get(&gbar, (size_t)N_s * rmax));
+        PTTK_TRY(sc.get(&gnext, (size_t)N_s * rmax));
+        PTTK_TRY(sc.get(&Q, (size_t)N_s * qmax));
+      }
+      for (int i = d - 1; i >= 0; --i) {
+        oriented_core_dims(tt, true, i, &rin, &rout, &coord);
+        const double lo = tt->box[coord][0], hi = tt->box[coord][1];
+        const int K = n * rin;
+        if (i < d - 1) {
+          const T* Gs = static_cast<const T*>(oriented_core_ptr(tt, true, i, fp64));
+          dim3 grid((unsigned)((K + 63) / 64), (unsigned)((N_s + 63) / 64));
+          gemm_gbar_core<T><<<grid, 256, 0, s>>>(gbar, Gs, N_s, rout, K, Q); pttk::count_launch();
+        }
+        const size_t smem = sizeof(T) * 8 * (PTTK_MAX_N + rin);
+        chain_back_step<T><<<(unsigned)((N_s + 7) / 8), 256, smem, s>>>(
+            X, d, coord, lo, hi, n, N_s, rin, i > 0 ? Sbuf[i] : nullptr, i < d - 1 ? Q : nullptr, w,
+            i == d - 1 ? q : nullptr, i > 0 ? gnext : nullptr, dX); pttk::count_launch();
+        std::swap(gbar, gnext);
+      }
     }
   }
   PTTK_CUDA(cudaGetLastError());

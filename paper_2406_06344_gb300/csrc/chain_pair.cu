@@ -80,14 +80,6 @@ struct PairArgs {
   uint32_t b_slot;
 };
 
-// One lane of the converged MMA warp: with the branch on elect.sync, unlike one on the lane number, the
-// compiler keeps the operands of tcgen05.mma in uniform registers. Alone on an SM an MMA then takes
-// 32 clocks at N = 64 and 96 at N = 192 (its tensor time), against 65 at N <= 64 from a lane branch.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
-  return r != 0;
-}
 __device__ __forceinline__ void pair_umma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"

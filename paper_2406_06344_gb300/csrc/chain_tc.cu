@@ -666,54 +666,64 @@ __global__ void __launch_bounds__(TCE_THREADS, 1) chain_tce_kernel(TcArgs a) {
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // the whole warp waits, one elected lane issues (see elect_one): the operands stay in uniform registers
+    {
+      const bool lead = elect_one();
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+      const uint32_t a_smem = __shfl_sync(0xffffffffu, smem_u32(a_base), 0);
+      const uint32_t b_smem = __shfl_sync(0xffffffffu, smem_u32(b_base), 0);
       uint32_t g = 0, tile = 0;
       bool ok = true;
       for (int64_t it = blockIdx.x; it < ntiles && ok; it += gridDim.x, ++tile) {
         const int sd = it >= a.T0 ? 1 : 0;
         const uint32_t r = tile & 1, use = tile >> 1;
         // the region's previous tile must have left it
-        if (use >= 1 && !mbar_wait(&rfree[r], (use - 1) & 1, abort_flag)) { ok = false; break; }
+        ok = use < 1 || mbar_wait(&rfree[r], (use - 1) & 1, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t dacc = region_addr(r);
+        const uint32_t dacc = tm + (r ? (uint32_t)a.region_col : 0u);
         for (int si = 0; si < nsteps && ok; ++si) {
-          const StepS& st = steps[sd * 3 + si];
-          for (int c = 0; c < st.nchunks; ++c, ++g) {
+          const uint32_t idesc = instr_desc(fmt_code(FMT), TILE_M, a.st[sd][si].Npad);
+          const int nchunks = a.st[sd][si].nchunks;
+          for (int c = 0; c < nchunks; ++c, ++g) {
             const uint32_t slot = g % NSLOT, par = (g / NSLOT) & 1;
-            if (!mbar_wait(&full_a[slot], par, abort_flag) || !mbar_wait(&full_b[slot], par, abort_flag)) {
-              ok = false;
-              break;
-            }
+            ok = mbar_wait(&full_a[slot], par, abort_flag) && mbar_wait(&full_b[slot], par, abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t sa = smem_u32(a_base + (size_t)slot * C::PARTS * C::A_PART);
-            const uint32_t sb = smem_u32(b_base + (size_t)slot * C::PARTS * a.b_slot_bytes);
+            const uint32_t sa = a_smem + slot * (C::PARTS * C::A_PART);
+            const uint32_t sb = b_smem + slot * C::PARTS * a.b_slot_bytes;
             const uint64_t ah0 = smem_desc2(sa, C::SBO), al0 = smem_desc2(sa + C::A_PART, C::SBO);
             const uint64_t bh0 = smem_desc2(sb, C::SBO), bl0 = smem_desc2(sb + a.b_slot_bytes, C::SBO);
+            if (lead) {
 #pragma unroll
             for (int k = 0; k < C::KSTEPS; ++k) {
               const uint32_t acc = (c > 0 || k > 0) ? 1u : 0u;
               // +256 bytes of K per MMA: +16 in the descriptors' address fields
               const uint64_t ah = ah0 + (uint64_t)(16 * k), bh = bh0 + (uint64_t)(16 * k);
               if constexpr (FMT != FMT_TF32) {
-                umma_f16(dacc, ah, bh, st.idesc, acc);
+                umma_f16(dacc, ah, bh, idesc, acc);
                 if (SPLIT) {
-                  umma_f16(dacc, ah, bl0 + (uint64_t)(16 * k), st.idesc, 1u);
-                  umma_f16(dacc, al0 + (uint64_t)(16 * k), bh, st.idesc, 1u);
+                  umma_f16(dacc, ah, bl0 + (uint64_t)(16 * k), idesc, 1u);
+                  umma_f16(dacc, al0 + (uint64_t)(16 * k), bh, idesc, 1u);
                 }
               } else {
-                umma_tf32(dacc, ah, bh, st.idesc, acc);
+                umma_tf32(dacc, ah, bh, idesc, acc);
                 if (SPLIT) {
-                  umma_tf32(dacc, ah, bl0 + (uint64_t)(16 * k), st.idesc, 1u);
-                  umma_tf32(dacc, al0 + (uint64_t)(16 * k), bh, st.idesc, 1u);
+                  umma_tf32(dacc, ah, bl0 + (uint64_t)(16 * k), idesc, 1u);
+                  umma_tf32(dacc, al0 + (uint64_t)(16 * k), bh, idesc, 1u);
                 }
               }
             }
             umma_commit(&empty[slot]);
-            if (c == st.nchunks - 1) umma_commit(si == nsteps - 1 ? &last_done[r] : &mid[r]);
+            if (c == nchunks - 1) umma_commit(si == nsteps - 1 ? &last_done[r] : &mid[r]);
+            }
+            __syncwarp();
           }
         }
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         *abort_flag = 1;
         atomicExch(a.status, (int)PTTK_ETIMEOUT);
       }

@@ -154,6 +154,14 @@ __device__ __forceinline__ float to_tf32(float x) {
   return __uint_as_float(r);
 }
 
+// One lane of the converged MMA warp: with the branch on elect.sync, unlike one on the lane number, the
+// compiler keeps the operands of tcgen05.mma in uniform registers. Alone on an SM an MMA then takes
+// 32 clocks at N = 64 and 96 at N = 192 (its tensor time), against 65 at N <= 64 from a lane branch.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+  return r != 0;
+}
 // UMMA shared-memory descriptor: no swizzle, K-major; K-adjacent core matrices 128 B apart
 // (leading byte offset), 8-row groups `sbo` bytes apart (stride byte offset).
 __device__ __forceinline__ uint64_t smem_desc2(uint32_t saddr, uint32_t sbo) {
