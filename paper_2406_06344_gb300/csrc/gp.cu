@@ -3,10 +3,10 @@
 // PTTK-Global factorisation (Algorithm 4), with the kernel matrix applied exactly.
 //
 //   pttk_gp_kv   out = (K(X, X; theta) + s2 I) v, every kernel entry evaluated on the fly
-//                (tiles of the points in shared memory; N^2 evaluations, no N x N storage), in
-//                FP64, or in FP32 with each tile's 128 terms summed in FP32 and the tile sums
-//                in FP64. Rows and column ranges are split over blocks so that small N fills
-//                the GPU; the column ranges' partial sums are added in a fixed order.
+//                (tiles of the points in shared memory, no N x N storage). In FP64 each unordered
+//                pair is evaluated once (gp_kv_sym_kernel); in FP32 (gp_kv_kernel, N^2
+//                evaluations) each tile's 128 terms are summed in FP32 and the tile sums in FP64.
+//                The tiles' partial sums are added in a fixed order.
 //   pttk_gp_pcg  preconditioned CG (Hestenes-Stiefel) with M^{-1} = (Z W Z^T + s2 I)^{-1},
 //                Z (N x m) with orthonormal columns and W = diag(lambda) (PTTK-Global-2, or
 //                Global-1 written in its eigenbasis), applied in Woodbury form
@@ -16,6 +16,7 @@
 #include <cmath>
 #include <vector>
 
+#include "fexp.cuh"
 #include "kernels.cuh"
 #include "pttk_internal.cuh"
 
@@ -61,6 +62,102 @@ __global__ void __launch_bounds__(GT) gp_kv_kernel(int kind, int d, const double
     }
   }
   if (i < N) part[(int64_t)blockIdx.y * N + i] = acc;
+}
+
+// Constants of one product: r^2 times `s` is the argument of the table exponential (Gaussian), or
+// `c` / l times r the decay's (the others).
+struct KvArgs {
+  double l, s, cl;
+  double r2max;  // Gaussian: r^2 up to which the table form holds (value above 2^-1010)
+};
+
+// kappa from r^2, with the table exponential: 6 (Gaussian) to about 25 FP64 operations in place of the 30 to 45 of
+// a division, CUDA's square root and exponential.
+__device__ __forceinline__ double kappa_fast(int kind, double r2, const KvArgs& k, const double* __restrict__ tab) {
+  if (kind == PTTK_GAUSS) {
+    // r2 s is 64 log2 of the value; beyond r2max, and for NaN, CUDA's exp decides
+    if ((unsigned)__double2hiint(r2) >= (unsigned)__double2hiint(k.r2max)) return exp(-r2 / (k.l * k.l));
+    return fexp2_64(r2, k.s, tab);
+  }
+  const double a = k.cl * sqrt(r2);
+  const double e = fexp_neg(a, tab);
+  if (kind == PTTK_MATERN32) return fma(a, e, e);
+  if (kind == PTTK_EXPONENTIAL) return e;
+  return fma(a * a, 1.0 / 3.0, 1.0 + a) * e;  // Matern-5/2
+}
+
+// K is symmetric, so each pair of points is evaluated once and used for both rows. A block takes the super
+// tile (I, J), J >= I, of S x S points in tiles of T x T: a thread holds one row, a warp goes through 32
+// columns in 32 steps in which lane t takes column (t + step) mod 32, and the column sums travel from lane
+// to lane with their columns (two shuffles, no extra FP64 operation). Row sums leave as part[J][i], column
+// sums (over the warps in shared memory) as part[I][j]; a diagonal super tile writes both together. Each entry of
+// part is written once, so the result does not depend on scheduling.
+// What bounds it: the FP64 pipe, 17 operations a pair for the Gaussian in d = 3. N = 20,000: 26.0 ms with every
+// ordered pair evaluated through CUDA's exp and a division, 5.9 ms so.
+template <int D, int T>
+__global__ void __launch_bounds__(T) gp_kv_sym_kernel(int kind, const double* __restrict__ X, int64_t N, KvArgs k, int S,
+                                                      int nS, const double* __restrict__ v, double* __restrict__ part) {
+  constexpr int W = T / 32;
+  extern __shared__ __align__(16) double col[];  // S column sums
+  __shared__ double tab[FEXP_N], xs[D][T], vs[T], cw[W][T];
+  // block -> (I, J): row I of the upper triangle holds nS - I blocks
+  int64_t b = blockIdx.x;
+  int I = (int)((2.0 * nS + 1.0 - sqrt((2.0 * nS + 1.0) * (2.0 * nS + 1.0) - 8.0 * (double)b)) * 0.5);
+  while ((int64_t)I * nS - (int64_t)I * (I - 1) / 2 > b) --I;
+  while ((int64_t)(I + 1) * nS - (int64_t)(I + 1) * I / 2 <= b) ++I;
+  const int J = I + (int)(b - ((int64_t)I * nS - (int64_t)I * (I - 1) / 2));
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int64_t i0 = (int64_t)I * S, j0 = (int64_t)J * S;
+  fexp_fill(tab);
+  for (int q = t; q < S; q += T) col[q] = 0.0;
+  for (int r = 0; r < S && i0 + r < N; r += T) {
+    const int64_t i = i0 + r + t;
+    double xi[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) xi[c] = i < N ? X[i * D + c] : 0.0;
+    const double vi = i < N ? v[i] : 0.0;
+    double acc = 0.0;
+    for (int c0 = I == J ? r : 0; c0 < S && j0 + c0 < N; c0 += T) {
+      const int64_t j = j0 + c0 + t;
+      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < D; ++c) xs[c][t] = j < N ? X[j * D + c] : 0.0;
+      vs[t] = j < N ? v[j] : 0.0;
+      __syncthreads();
+      const bool diag = I == J && c0 == r;
+      for (int g = 0; g < W; ++g) {
+        double cacc = 0.0;
+#pragma unroll 2
+        for (int step = 0; step < 32; ++step) {
+          const int jj = 32 * g + ((lane + step) & 31);
+          double r2 = 0.0;
+#pragma unroll
+          for (int c = 0; c < D; ++c) {
+            const double df = xi[c] - xs[c][jj];
+            r2 = fma(df, df, r2);
+          }
+          const double kv = kappa_fast(kind, r2, k, tab);
+          acc = fma(kv, vs[jj], acc);
+          if (!diag) {
+            cacc = fma(kv, vi, cacc);
+            cacc = __shfl_sync(0xffffffffu, cacc, lane + 1);
+          }
+        }
+        if (!diag) cw[w][32 * g + lane] = cacc;
+      }
+      if (!diag) {
+        __syncthreads();
+        double sum = 0.0;
+#pragma unroll
+        for (int q = 0; q < W; ++q) sum += cw[q][t];
+        col[c0 + t] += sum;
+      }
+    }
+    if (i < N) part[(int64_t)J * N + i] = I == J ? acc + col[r + t] : acc;
+  }
+  if (I != J)
+    for (int q = t; q < S; q += T)
+      if (j0 + q < N) part[(int64_t)I * N + j0 + q] = col[q];
 }
 
 // out[i] = s2 v[i] + sum over the column ranges of part (in order)
@@ -164,22 +261,79 @@ unsigned grid_for(int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + GT - 1) / GT, (int64_t)sm_count() * 8));
 }
 
-// column ranges of the kernel product: enough blocks for about four per SM
+// Tile and super-tile edge of the symmetric product: 256-point tiles, 64-point ones where those would give
+// fewer than four blocks per SM; super tiles of as many tiles as keep the partial sums at 96 N.
+void kv_sym_shape(int64_t N, int* T, int* S, int* nS) {
+  const int64_t t256 = (N + 255) / 256;
+  *T = t256 * (t256 + 1) / 2 >= (int64_t)sm_count() * 4 ? 256 : 64;
+  const int64_t tiles = (N + *T - 1) / *T;
+  const int64_t per = (tiles + 95) / 96;
+  *S = (int)(per * *T);
+  *nS = (int)((N + *S - 1) / *S);
+}
+
+// column ranges of gp_kv_kernel: enough blocks for about four per SM
 int kv_splits(int64_t N) {
   const int64_t row_tiles = (N + GT - 1) / GT;
   const int64_t want = std::max<int64_t>(1, (int64_t)sm_count() * 4 / std::max<int64_t>(row_tiles, 1));
   return (int)std::min<int64_t>({want, 64, (N + GTILE - 1) / GTILE});
 }
 
-// out = (K + s2 I) v; part: scratch of kv_splits(N) * N doubles
+// The symmetric form serves FP64 products up to about 2.3 million points (its column sums in shared memory).
+bool kv_symmetric(int64_t N, bool fp32) {
+  int T, S, nS;
+  kv_sym_shape(N, &T, &S, &nS);
+  return !fp32 && S <= 24576;
+}
+
+// doubles of scratch for one product
+size_t kv_part_elems(int64_t N, bool fp32) {
+  if (!kv_symmetric(N, fp32)) return (size_t)kv_splits(N) * N;
+  int T, S, nS;
+  kv_sym_shape(N, &T, &S, &nS);
+  return (size_t)nS * N;
+}
+
+template <int D>
+pttk_status kv_sym_launch(int kind, const double* X, int64_t N, const KvArgs& k, const double* v, double* part,
+                          cudaStream_t s) {
+  int T, S, nS;
+  kv_sym_shape(N, &T, &S, &nS);
+  const unsigned blocks = (unsigned)((int64_t)nS * (nS + 1) / 2);
+  const size_t smem = sizeof(double) * S;
+  auto kfn = T == 256 ? gp_kv_sym_kernel<D, 256> : gp_kv_sym_kernel<D, 64>;
+  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kfn<<<blocks, T, smem, s>>>(kind, X, N, k, S, nS, v, part);
+  return PTTK_OK;
+}
+
+// out = (K + s2 I) v; part: scratch of kv_part_elems(N, fp32) doubles
 pttk_status kv_launch(int kind, int d, const double* X, int64_t N, double l, double s2, const double* v, double* out,
                       bool fp32, double* part, cudaStream_t s) {
   PTTK_PROF("gp_kv", s);
-  const int ncs = kv_splits(N);
-  const int64_t cols = ((N + ncs - 1) / ncs + GTILE - 1) / GTILE * GTILE;
-  const dim3 grid((unsigned)((N + GT - 1) / GT), (unsigned)ncs);
-  if (fp32) gp_kv_kernel<float><<<grid, GT, 0, s>>>(kind, d, X, N, l, v, cols, part);
-  else gp_kv_kernel<double><<<grid, GT, 0, s>>>(kind, d, X, N, l, v, cols, part);
+  int ncs;
+  if (!kv_symmetric(N, fp32)) {
+    ncs = kv_splits(N);
+    const int64_t cols = ((N + ncs - 1) / ncs + GTILE - 1) / GTILE * GTILE;
+    const dim3 grid((unsigned)((N + GT - 1) / GT), (unsigned)ncs);
+    if (fp32) gp_kv_kernel<float><<<grid, GT, 0, s>>>(kind, d, X, N, l, v, cols, part);
+    else gp_kv_kernel<double><<<grid, GT, 0, s>>>(kind, d, X, N, l, v, cols, part);
+  } else {
+    int T, S;
+    kv_sym_shape(N, &T, &S, &ncs);
+    const double c = kind == PTTK_MATERN32 ? 1.7320508075688772 : kind == PTTK_MATERN52 ? 2.23606797749979 : 1.0;
+    const KvArgs k{l, -64.0 / (0.69314718055994530942 * l * l), c / l, 1010.0 * 0.69314718055994530942 * l * l};
+    switch (d) {
+      case 1: PTTK_TRY(kv_sym_launch<1>(kind, X, N, k, v, part, s)); break;
+      case 2: PTTK_TRY(kv_sym_launch<2>(kind, X, N, k, v, part, s)); break;
+      case 3: PTTK_TRY(kv_sym_launch<3>(kind, X, N, k, v, part, s)); break;
+      case 4: PTTK_TRY(kv_sym_launch<4>(kind, X, N, k, v, part, s)); break;
+      case 5: PTTK_TRY(kv_sym_launch<5>(kind, X, N, k, v, part, s)); break;
+      case 6: PTTK_TRY(kv_sym_launch<6>(kind, X, N, k, v, part, s)); break;
+      case 7: PTTK_TRY(kv_sym_launch<7>(kind, X, N, k, v, part, s)); break;
+      default: PTTK_TRY(kv_sym_launch<8>(kind, X, N, k, v, part, s)); break;
+    }
+  }
   pttk::count_launch();
   gp_kv_reduce<<<grid_for(N), GT, 0, s>>>(part, ncs, N, s2, v, out); pttk::count_launch();
   PTTK_CUDA(cudaGetLastError());
@@ -226,7 +380,7 @@ pttk_status pttk_gp_kv(int kernel, int d, const double* X, int64_t N, const doub
   if (prec != PTTK_FP64 && prec != PTTK_FP32) return set_error(PTTK_EINVAL, "K v: prec must be PTTK_FP64 or PTTK_FP32");
   cudaStream_t s = as_stream(stream);
   double* part = nullptr;
-  PTTK_CUDA(ws_malloc(&part, sizeof(double) * (size_t)kv_splits(N) * N, s));
+  PTTK_CUDA(ws_malloc(&part, sizeof(double) * kv_part_elems(N, prec == PTTK_FP32), s));
   const pttk_status st = kv_launch(kernel, d, X, N, theta[0], s2, v, out, prec == PTTK_FP32, part, s);
   cudaFreeAsync(part, s);
   return st;
@@ -253,7 +407,7 @@ pttk_status pttk_gp_pcg(int kernel, int d, const double* X, int64_t N, const dou
   PTTK_TRY(sc.get(&Ap, N));
   PTTK_TRY(sc.get(&part, nparts));
   double* kvpart = nullptr;
-  PTTK_TRY(sc.get(&kvpart, (size_t)kv_splits(N) * N));
+  PTTK_TRY(sc.get(&kvpart, kv_part_elems(N, prec == PTTK_FP32)));
   if (m > 0) {
     PTTK_TRY(sc.get(&coef, m));
     PTTK_TRY(sc.get(&gpart, (size_t)gparts * m));
