@@ -36,7 +36,11 @@ def test_folded_coefficients(kernel, d, n, src, tgt, prec, tol):
     D = 2 * d + dth
     C = C.reshape((n,) * D, order="F")
     boxes = np.array(list(src) + list(theta) + list(tgt))
-    ref = o.coefficient_tensor(o.grid_tensor(o.kernel_f(kernel), d, dth, boxes, n), n)
+    with np.errstate(invalid="ignore"):
+        M = o.grid_tensor(o.kernel_f(kernel), d, dth, boxes, n)
+    if kernel == W.MATERN_NU:
+        M = np.where(np.isnan(M), 1.0, M)   # the oracle's z^nu K_nu(z) at z = 0, whose limit gives kappa = 1
+    ref = o.coefficient_tensor(M, n)
     assert np.abs(C - ref).max() <= tol * np.abs(ref).max()
     for j in range(d):
         if sum(src[j]) == sum(tgt[j]):
