@@ -93,7 +93,7 @@ __device__ __forceinline__ double kappa_fast(int kind, double r2, const KvArgs& 
 // sums (over the warps in shared memory) as part[I][j]; a diagonal super tile writes both together. Each entry of
 // part is written once, so the result does not depend on scheduling.
 // What bounds it: the FP64 pipe, 17 operations a pair for the Gaussian in d = 3. N = 20,000: 26.0 ms with every
-// ordered pair evaluated through CUDA's exp and a division, 5.9 ms so.
+// ordered pair evaluated through CUDA's exp and a division, 6.5 ms so.
 template <int D, int T>
 __global__ void __launch_bounds__(T) gp_kv_sym_kernel(int kind, const double* __restrict__ X, int64_t N, KvArgs k, int S,
                                                       int nS, const double* __restrict__ v, double* __restrict__ part) {

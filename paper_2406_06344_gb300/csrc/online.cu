@@ -48,33 +48,36 @@ template <>
 __device__ __forceinline__ float warp_sum<float>(float v) { return warp_sum_f(v); }
 
 // ---------------- H(theta) -------------------------------------------------------------
-// out[a + ra b] = sum_k G[a + ra (k + n b)] T_k(th)   (G: ra x n x rb, column-major)
-__global__ void contract_theta_kernel(const double* __restrict__ G, int ra, int n, int rb,
-                                      double th, double* __restrict__ out) {
-  double T[PTTK_MAX_N];
-  T[0] = 1.0;
-  if (n > 1) T[1] = th;
-  for (int k = 2; k < n; ++k) T[k] = 2.0 * th * T[k - 1] - T[k - 2];
+// One or two theta cores contracted with their Chebyshev vectors in one launch (blockIdx.y: the core), G
+// (ra x n x rb, column-major): sum_k G[a + ra (k + n b)] T_k(th), into out[a + ra b], or, for a single core, row-major
+// into M.
+struct ThetaCores {
+  const double* G[2];
+  double* out[2];
+  double th[2];
+  int ra[2], rb[2];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) contract_theta_kernel(ThetaCores c, int n, T* __restrict__ M) {
+  const int q = blockIdx.y;
+  const double* __restrict__ G = c.G[q];
+  const int ra = c.ra[q], rb = c.rb[q];
+  const double th = c.th[q];
   const int64_t total = (int64_t)ra * rb;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t a = e % ra, b = e / ra;
+    const int a = (int)(e % ra), b = (int)(e / ra);
     const double* g = G + a + (int64_t)ra * n * b;
-    double acc = 0.0;
-    for (int k = 0; k < n; ++k) acc = fma(g[(int64_t)ra * k], T[k], acc);
-    out[e] = acc;
-  }
-}
-
-// M row-major (rs x rt) from H column-major (rs x rt)
-template <typename T>
-__global__ void store_rowmajor_kernel(const double* __restrict__ H, int rs, int rt,
-                                      T* __restrict__ M) {
-  const int64_t total = (int64_t)rs * rt;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t a = e / rt, b = e % rt;
-    M[e] = (T)H[a + (int64_t)rs * b];
+    double t0 = 1.0, t1 = th, acc = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+      acc = fma(g[(int64_t)ra * k], t0, acc);
+      const double t2 = 2.0 * th * t1 - t0;
+      t0 = t1;
+      t1 = t2;
+    }
+    if (M) M[(int64_t)a * rb + b] = (T)acc;
+    else c.out[q][e] = acc;
   }
 }
 
@@ -278,7 +281,7 @@ __device__ void chain_step_narrow(const ChainStep& st, int n, const T* __restric
 
 // Factor rows of both sides: a block takes 16 TM points of one side. TM is chosen by the point counts and
 // ranks (factor_build_run). What bounds it: FMA issue. 200k points a side, ranks 10, 63 | 63, 12, n = 20:
-// FP32 1.156 -> 0.29 ms, FP64 11.13 -> 9.9 ms (9.05 ms at the DFMA rate), against 64 points x 64 columns a
+// FP32 1.156 -> 0.457 ms, FP64 11.13 -> 10.20 ms (9.05 ms at the DFMA rate), against 64 points x 64 columns a
 // block, 4 x 4 a thread, one buffer and a tiled first step.
 template <typename T, int TM>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) chain_kernel(ChainArgs a) {
@@ -329,66 +332,87 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) chain_kernel(Chai
 }
 
 // ---------------- apply: out = U (M (V^T w)) ----------------------------------------
-// partial[b, c] = sum over block b's rows r of V[r, c] w[r]. Threads are 4 row lanes x 64
-// column groups, each of VW consecutive columns (VW = 4 when rows are 16-byte aligned: a row
-// of up to 256 columns is then read once, contiguously, by 16-byte loads; else VW = 1 and 64
-// columns a pass). Each thread keeps 4 rows of loads in flight; the row lanes meet in shared
-// memory in a fixed order.
+// partial[b, c] = sum over block b's rows r of V[r, c] w[r], V read as a flat array of 16-byte units (of
+// VW elements, whatever rt is): a unit of P rows (P rt a multiple of VW) always covers the same columns, so thread t
+// keeps VW accumulators, whose column and row offset never change, and takes unit t of every group of P rows;
+// nt = P rt / VW threads make a group, and as many groups as fit run side by side, UNR of them in flight per thread.
+// The accumulators of a column meet in shared memory in a fixed order. (V not 16-byte aligned: VW = 1, P = 1.)
+// What bounds it: the read of V (2.6 TB/s from L2 at this size). 100k x 180 FP32: 34 -> 28 us; 100k x 63 FP64, where a
+// unit holds two columns: 19 -> 22 us, beside a 10 ms chain.
 template <typename T, int VW>
 __global__ void __launch_bounds__(256) vtw_partial_kernel(const T* __restrict__ V, int64_t N,
-                                                          int rt, const T* __restrict__ w,
+                                                          int rt, int P, const T* __restrict__ w,
                                                           T* __restrict__ partial) {
-  __shared__ T red[4][64 * VW];
-  const int64_t rows_per = (N + gridDim.x - 1) / gridDim.x;
-  const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = std::min<int64_t>(N, r0 + rows_per);
-  const int cl = threadIdx.x & 63, rl = threadIdx.x >> 6;
-  for (int cb = 0; cb < rt; cb += 64 * VW) {
-    const int c = cb + cl * VW;
-    const bool on = c < rt;  // with VW = 4, rt is a multiple of 4: the whole group is in range
+  constexpr int UNR = 4;
+  __shared__ T red[256 * VW];
+  const int nt = P * rt / VW;
+  const int64_t groups = (N + P - 1) / P;
+  const int64_t per = (groups + gridDim.x - 1) / gridDim.x;
+  const int64_t g0 = (int64_t)blockIdx.x * per, g1 = std::min<int64_t>(groups, g0 + per);
+  for (int tb = 0; tb < nt; tb += 256) {  // more than 256 units a group: one pass per 256
+    const int width = std::min(256, nt - tb), lanes = 256 / width;
+    const int t = tb + threadIdx.x % width, gl = threadIdx.x / width;
+    const bool on = gl < lanes;
+    int off[VW];
     T acc[VW];
 #pragma unroll
-    for (int q = 0; q < VW; ++q) acc[q] = T(0);
-    int64_t r = r0 + rl;
-    for (; r + 12 < r1; r += 16) {
-      T v[4][VW];
+    for (int e = 0; e < VW; ++e) {
+      off[e] = (VW * t + e) / rt;
+      acc[e] = T(0);
+    }
+    auto load = [&](int64_t g, T* v) {
+      const T* src = V + g * P * rt + (int64_t)VW * t;
+      if constexpr (VW == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(src);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+      } else if constexpr (VW == 2) {
+        const double2 x = *reinterpret_cast<const double2*>(src);
+        v[0] = x.x; v[1] = x.y;
+      } else {
+        v[0] = *src;
+      }
+    };
+    if (on) {
+      // groups that lie wholly inside N; the last one may not
+      const int64_t gfull = std::min<int64_t>(g1, N / P);
+      int64_t g = g0 + gl;
+      for (; g + (UNR - 1) * lanes < gfull; g += UNR * lanes) {
+        T v[UNR][VW];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const T* src = V + (r + 4 * u) * rt + c;
-        if constexpr (VW == 4) {
-          if (on) {
-            if constexpr (sizeof(T) == 4) {
-              const float4 x = *reinterpret_cast<const float4*>(src);
-              v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
-            } else {
-              const double2 x0 = *reinterpret_cast<const double2*>(src);
-              const double2 x1 = *reinterpret_cast<const double2*>(src + 2);
-              v[u][0] = x0.x; v[u][1] = x0.y; v[u][2] = x1.x; v[u][3] = x1.y;
-            }
-          } else {
+        for (int u = 0; u < UNR; ++u) load(g + u * lanes, v[u]);
 #pragma unroll
-            for (int q = 0; q < VW; ++q) v[u][q] = T(0);
-          }
-        } else {
-          v[u][0] = on ? *src : T(0);
+        for (int u = 0; u < UNR; ++u)
+#pragma unroll
+          for (int e = 0; e < VW; ++e) acc[e] = fma(v[u][e], w[(g + u * lanes) * P + off[e]], acc[e]);
+      }
+      for (; g < gfull; g += lanes) {
+        T v[VW];
+        load(g, v);
+#pragma unroll
+        for (int e = 0; e < VW; ++e) acc[e] = fma(v[e], w[g * P + off[e]], acc[e]);
+      }
+      if (g < g1)
+#pragma unroll
+        for (int e = 0; e < VW; ++e) {
+          const int64_t row = g * P + off[e];
+          if (row < N) acc[e] = fma(V[g * P * rt + (int64_t)VW * t + e], w[row], acc[e]);
         }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const T wr = w[r + 4 * u];
-#pragma unroll
-        for (int q = 0; q < VW; ++q) acc[q] = fma(v[u][q], wr, acc[q]);
-      }
     }
-    for (; r < r1; r += 4) {
-      const T wr = w[r];
-#pragma unroll
-      for (int q = 0; q < VW; ++q) acc[q] = fma(on ? V[r * rt + c + q] : T(0), wr, acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < VW; ++q) red[rl][cl * VW + q] = acc[q];
     __syncthreads();
-    for (int q = threadIdx.x; q < 64 * VW; q += blockDim.x)
-      if (cb + q < rt) partial[(int64_t)blockIdx.x * rt + cb + q] = (red[0][q] + red[1][q]) + (red[2][q] + red[3][q]);
+#pragma unroll
+    for (int e = 0; e < VW; ++e) red[threadIdx.x * VW + e] = acc[e];
+    __syncthreads();
+    // element VW t + e of a group is column (VW t + e) mod rt; red holds elements VW tb .. of every lane
+    for (int c = threadIdx.x; c < rt; c += 256) {
+      T sum = T(0);
+      for (int el = c; el < P * rt; el += rt) {
+        const int q = el - VW * tb;
+        if (q < 0 || q >= VW * width) continue;
+        for (int l = 0; l < lanes; ++l) sum += red[(l * width) * VW + q];
+      }
+      T* dst = partial + (int64_t)blockIdx.x * rt + c;
+      *dst = tb == 0 ? sum : *dst + sum;
+    }
     __syncthreads();
   }
 }
@@ -411,46 +435,67 @@ __global__ void __launch_bounds__(256) reduce_parts_kernel(T* __restrict__ parti
                  ((red[4][cl] + red[5][cl]) + (red[6][cl] + red[7][cl]));
 }
 
-// s = M t, one warp per row of M (rs x rt, row-major); t is read through the L1 cache, so
-// no shared memory is sized by a rank.
+// s = M t, one warp per row of M (rs x rt, row-major); t is the sum of the nparts rows of `partial` (one row
+// once reduce_parts_kernel has run; a few where the sum is cheaper than that launch), formed by
+// each block in shared memory 1024 columns at a time.
 template <typename T>
 __global__ void __launch_bounds__(256) mt_kernel(const T* __restrict__ M, int rs, int rt,
-                                                 const T* __restrict__ t, T* __restrict__ s_out) {
+                                                 const T* __restrict__ partial, int nparts, T* __restrict__ s_out) {
+  __shared__ T t[1024];
   const int lane = threadIdx.x & 31;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rs;
-       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const T* m = M + r * rt;
-    T acc = T(0);
-    for (int c = lane; c < rt; c += 32) acc = fma(m[c], __ldg(t + c), acc);
-    acc = warp_sum<T>(acc);
-    if (lane == 0) s_out[r] = acc;
+  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  T acc = T(0);
+  for (int c0 = 0; c0 < rt; c0 += 1024) {
+    const int w = std::min(1024, rt - c0);
+    __syncthreads();
+    for (int c = threadIdx.x; c < w; c += 256) {
+      T sum = T(0);
+      for (int b = 0; b < nparts; ++b) sum += partial[(int64_t)b * rt + c0 + c];
+      t[c] = sum;
+    }
+    __syncthreads();
+    if (r < rs) {
+      const T* m = M + r * rt + c0;
+      for (int c = lane; c < w; c += 32) acc = fma(m[c], t[c], acc);
+    }
   }
+  acc = warp_sum<T>(acc);
+  if (lane == 0 && r < rs) s_out[r] = acc;
 }
 
-// out[p] = U[p, :] . s, one warp per row, two rows at a time (the loads of both are in
-// flight before either is reduced); s is read through the L1 cache
+// out[p] = U[p, :] . s, a warp taking four consecutive rows at a time (their loads are all in
+// flight before any is reduced); s is read through the L1 cache. What bounds it: the read of U.
+// 100k x 177 FP32: 24.3 -> 18.8 us, 200k x 63: 23 -> 14.9 us, against one row at a time.
 template <typename T>
 __global__ void __launch_bounds__(256) us_kernel(const T* __restrict__ U, int64_t N, int rs,
                                                  const T* __restrict__ s, T* __restrict__ out) {
+  constexpr int R = 4;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < N; row += 2 * nw) {
-    const int64_t row2 = row + nw;
-    const bool two = row2 < N;
+  for (int64_t row = R * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); row < N; row += R * nw) {
+    const int live = (int)std::min<int64_t>(R, N - row);
     const T* u = U + row * rs;
-    const T* u2 = U + (two ? row2 : row) * rs;
-    T acc = T(0), acc2 = T(0);
-    for (int c = lane; c < rs; c += 32) {
-      const T sc = __ldg(s + c);
-      acc = fma(u[c], sc, acc);
-      acc2 = fma(u2[c], sc, acc2);
+    T acc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = T(0);
+    if (live == R) {
+#pragma unroll 4
+      for (int c = lane; c < rs; c += 32) {
+        const T sc = __ldg(s + c);
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i] = fma(u[(int64_t)i * rs + c], sc, acc[i]);
+      }
+    } else {
+      for (int c = lane; c < rs; c += 32) {
+        const T sc = __ldg(s + c);
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+          if (i < live) acc[i] = fma(u[(int64_t)i * rs + c], sc, acc[i]);
+      }
     }
-    acc = warp_sum<T>(acc);
-    acc2 = warp_sum<T>(acc2);
-    if (lane == 0) {
-      out[row] = acc;
-      if (two) out[row2] = acc2;
-    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = warp_sum<T>(acc[i]);
+    if (lane < live) out[row + lane] = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
   }
 }
 
@@ -461,21 +506,25 @@ pttk_status apply_typed(const T* U, const T* M, const T* V, int64_t N_s, int64_t
   T* sv = scratch + (size_t)nparts * rt;
   PTTK_PROF("apply", s);
   if (N_t > 0) {
-    // 16-byte column groups when every row starts on a 16-byte boundary
-    const bool vec = rt % 4 == 0 && (reinterpret_cast<uintptr_t>(V) & 15) == 0 && (sizeof(T) * rt) % 16 == 0;
-    if (vec) vtw_partial_kernel<T, 4><<<nparts, 256, 0, s>>>(V, N_t, rt, w, partial);
-    else vtw_partial_kernel<T, 1><<<nparts, 256, 0, s>>>(V, N_t, rt, w, partial);
+    constexpr int VW = 16 / (int)sizeof(T);
+    if ((reinterpret_cast<uintptr_t>(V) & 15) == 0) {
+      const int P = rt % VW == 0 ? 1 : VW % 2 == 0 && (2 * rt) % VW == 0 ? 2 : VW;
+      vtw_partial_kernel<T, VW><<<nparts, 256, 0, s>>>(V, N_t, rt, P, w, partial);
+    } else {
+      vtw_partial_kernel<T, 1><<<nparts, 256, 0, s>>>(V, N_t, rt, 1, w, partial);
+    }
     pttk::count_launch();
   } else {
     PTTK_CUDA(cudaMemsetAsync(partial, 0, sizeof(T) * (size_t)nparts * rt, s));
   }
-  if (nparts > 1) {
+  int left = nparts;
+  if (nparts > 32) {
     reduce_parts_kernel<T><<<(unsigned)((rt + 31) / 32), 256, 0, s>>>(partial, nparts, rt); pttk::count_launch();
+    left = 1;
   }
-  const int64_t mblocks = std::min<int64_t>(((int64_t)rs * 32 + 255) / 256, (int64_t)sm_count() * 16);
-  mt_kernel<T><<<(unsigned)mblocks, 256, 0, s>>>(M, rs, rt, partial, sv); pttk::count_launch();
+  mt_kernel<T><<<(unsigned)((rs + 7) / 8), 256, 0, s>>>(M, rs, rt, partial, left, sv); pttk::count_launch();
   if (N_s > 0) {
-    const int64_t blocks = std::min<int64_t>((N_s * 32 + 255) / 256, (int64_t)sm_count() * 16);
+    const int64_t blocks = std::min<int64_t>((N_s * 8 + 255) / 256, (int64_t)sm_count() * 8);
     us_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(U, N_s, rs, sv, out); pttk::count_launch();
   }
   PTTK_CUDA(cudaGetLastError());
@@ -663,35 +712,40 @@ pttk_status theta_core_run(const pttk_tt* tt, const double* theta_hat, bool fp64
     return PTTK_OK;
   }
   PTTK_PROF("theta_core", s);
+  ThetaCores c{};
+  int64_t most = 0;
+  for (int j = 0; j < dth; ++j) {
+    c.G[j] = tt->cores64 + tt->core_off[d + j];
+    c.th[j] = theta_hat[j];
+    c.ra[j] = tt->ranks[d + j];
+    c.rb[j] = tt->ranks[d + j + 1];
+    most = std::max(most, (int64_t)c.ra[j] * c.rb[j]);
+  }
+  const dim3 cgrid((unsigned)std::min<int64_t>((most + 255) / 256, sm_count() * 8), (unsigned)dth);
+  if (dth == 1) {
+    if (fp64) contract_theta_kernel<double><<<cgrid, 256, 0, s>>>(c, n, static_cast<double*>(M));
+    else contract_theta_kernel<float><<<cgrid, 256, 0, s>>>(c, n, static_cast<float*>(M));
+    pttk::count_launch();
+    PTTK_CUDA(cudaGetLastError());
+    return PTTK_OK;
+  }
   const int rm = tt->ranks[d + 1];
   const int nslices = (rm + HP_T - 1) / HP_T;
-  size_t need = 0;
-  for (int j = 0; j < dth; ++j) need += (size_t)tt->ranks[d + j] * tt->ranks[d + j + 1];
-  need += (size_t)rs * rt * (dth > 1 ? nslices : 0);
+  const size_t e1 = (size_t)rs * rm, e2 = (size_t)rm * rt;
   double* work = nullptr;
-  PTTK_CUDA(ws_malloc(&work, sizeof(double) * std::max<size_t>(need, 1), s));
-  double* Hj[2] = {work, work + (size_t)tt->ranks[d] * tt->ranks[d + 1]};
-  for (int j = 0; j < dth; ++j) {
-    const int ra = tt->ranks[d + j], rb = tt->ranks[d + j + 1];
-    const int64_t total = (int64_t)ra * rb;
-    const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, sm_count() * 8);
-    contract_theta_kernel<<<blocks, 256, 0, s>>>(tt->cores64 + tt->core_off[d + j], ra, n, rb,
-                                                 theta_hat[j], Hj[j]); pttk::count_launch();
-  }
+  PTTK_CUDA(ws_malloc(&work, sizeof(double) * (e1 + e2 + (size_t)rs * rt * nslices), s));
+  c.out[0] = work;
+  c.out[1] = work + e1;
+  double* part = work + e1 + e2;
+  contract_theta_kernel<double><<<cgrid, 256, 0, s>>>(c, n, nullptr); pttk::count_launch();
   const unsigned blocks = (unsigned)std::min<int64_t>(((int64_t)rs * rt + 255) / 256, sm_count() * 8);
-  if (dth == 2) {
-    double* part = Hj[1] + (size_t)rm * rt;
-    const dim3 grid((unsigned)((rs + HP_T - 1) / HP_T), (unsigned)((rt + HP_T - 1) / HP_T), (unsigned)nslices);
-    hprod_splitk_kernel<<<grid, 256, 0, s>>>(Hj[0], Hj[1], rs, rm, rt, part); pttk::count_launch();
-    if (fp64) { hprod_reduce_kernel<double><<<blocks, 256, 0, s>>>(part, nslices, rs, rt, static_cast<double*>(M)); pttk::count_launch(); }
-    else { hprod_reduce_kernel<float><<<blocks, 256, 0, s>>>(part, nslices, rs, rt, static_cast<float*>(M)); pttk::count_launch(); }
-  } else if (fp64) {
-    store_rowmajor_kernel<double><<<blocks, 256, 0, s>>>(Hj[0], rs, rt, static_cast<double*>(M)); pttk::count_launch();
-  } else {
-    store_rowmajor_kernel<float><<<blocks, 256, 0, s>>>(Hj[0], rs, rt, static_cast<float*>(M)); pttk::count_launch();
-  }
-  PTTK_CUDA(cudaGetLastError());
-  PTTK_CUDA(cudaFreeAsync(work, s));
+  const dim3 grid((unsigned)((rs + HP_T - 1) / HP_T), (unsigned)((rt + HP_T - 1) / HP_T), (unsigned)nslices);
+  hprod_splitk_kernel<<<grid, 256, 0, s>>>(c.out[0], c.out[1], rs, rm, rt, part); pttk::count_launch();
+  if (fp64) { hprod_reduce_kernel<double><<<blocks, 256, 0, s>>>(part, nslices, rs, rt, static_cast<double*>(M)); pttk::count_launch(); }
+  else { hprod_reduce_kernel<float><<<blocks, 256, 0, s>>>(part, nslices, rs, rt, static_cast<float*>(M)); pttk::count_launch(); }
+  const cudaError_t err = cudaGetLastError();
+  cudaFreeAsync(work, s);
+  PTTK_CUDA(err);
   return PTTK_OK;
 }
 

@@ -66,8 +66,8 @@ int sm_count();
 
 // Stream-ordered scratch (freed with cudaFreeAsync) from the library's own memory pool of the current
 // device. The default pool gives all memory back at every synchronisation, so a caller that reads
-// each result paid for the mapping again in each call (220 us in an instantiate + apply, about 4 ms
-// for the adjoint's factors at N = 500k); this one keeps up to kWorkspaceKeep bytes until the last
+// each result paid for the mapping again in each call (220 us in an instantiate +
+// apply); this one keeps up to kWorkspaceKeep bytes until the last
 // handle is freed. While the stream is being captured, the default pool's graph allocations serve.
 constexpr unsigned long long kWorkspaceKeep = 1ull << 30;
 cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s);
