@@ -183,7 +183,7 @@ template <typename T, int TM, int TN>
 __device__ void chain_step(const ChainStep& st, int n, const T* __restrict__ Bv, const T* __restrict__ Sin,
                            T* __restrict__ Sout, T* __restrict__ As, T* __restrict__ Gs, T* __restrict__ out, int64_t p0,
                            int64_t N, bool last) {
-  constexpr int P = 16 * TM, CT = 16 * TN, GL = CT + 4;
+  constexpr int P = 16 * TM, CT = 16 * TN, GL = CT + 2;
   constexpr int NA = BK * P / 256, NG = BK * CT / 256;
   const T* __restrict__ G = static_cast<const T*>(st.G);
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -281,10 +281,12 @@ __device__ void chain_step_narrow(const ChainStep& st, int n, const T* __restric
 
 // Factor rows of both sides: a block takes 16 TM points of one side. TM is chosen by the point counts and
 // ranks (factor_build_run). What bounds it: FMA issue. 200k points a side, ranks 10, 63 | 63, 12, n = 20:
-// FP32 1.156 -> 0.457 ms, FP64 11.13 -> 10.20 ms (9.05 ms at the DFMA rate), against 64 points x 64 columns a
+// FP32 1.156 -> 0.38 ms, FP64 11.13 -> 9.95 ms (9.05 ms at the DFMA rate), against 64 points x 64 columns a
 // block, 4 x 4 a thread, one buffer and a tiled first step.
-template <typename T, int TM>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) chain_kernel(ChainArgs a) {
+// CTMAX, the widest pass any step takes, sets the registers: FP32 up to 64 columns runs three blocks an SM (two:
+// 0.457 ms), all others two (FP64 with one: 10.25 ms).
+template <typename T, int TM, int CTMAX>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 && CTMAX == 64 ? 3 : 2) chain_kernel(ChainArgs a) {
   constexpr int P = 16 * TM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int sd = (int64_t)blockIdx.x < a.blocks0 ? 0 : 1;
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) chain_kernel(Chai
   T* Sout = Sin + (size_t)a.rin_max * P;
   T* Bv = Sout + (size_t)a.rin_max * P;         // n x P basis values
   T* As = Bv + (size_t)n * P;                   // 2 x BK x P
-  T* Gs = As + 2 * BK * P;                      // 2 x BK x (ct + 4)
+  T* Gs = As + 2 * BK * P;                      // 2 x BK x (ct + 2): the transposed stores of a core chunk meet the fewest bank conflicts
   const int64_t p0 = ((int64_t)blockIdx.x - (sd ? a.blocks0 : 0)) * P, N = side.N;
   const T* __restrict__ pts = static_cast<const T*>(side.pts);
   T* out = static_cast<T*>(side.out);
@@ -322,8 +324,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) chain_kernel(Chai
     switch (st.ct) {
       case 0: chain_step_narrow<T, P>(st, n, Bv, Sin, Sout, out, p0, N, last); break;
       case 64: chain_step<T, TM, 4>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
-      case 96: chain_step<T, TM, 6>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
-      default: chain_step<T, TM, 8>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
+      case 96: if constexpr (CTMAX >= 96) chain_step<T, TM, 6>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
+      default: if constexpr (CTMAX >= 128) chain_step<T, TM, 8>(st, n, Bv, Sin, Sout, As, Gs, out, p0, N, last); break;
     }
     T* tmp = Sin;
     Sin = Sout;
@@ -755,8 +757,8 @@ const void* oriented_core_ptr(const pttk_tt* tt, bool source, int k, bool fp64);
 template <typename T, int TM>
 static pttk_status launch_chain(ChainArgs a, int ct_max, cudaStream_t s) {
   constexpr int P = 16 * TM;
-  const size_t smem = sizeof(T) * ((size_t)2 * P * a.rin_max + (size_t)P * a.n + 2 * BK * P + 2 * BK * (ct_max + 4));
-  auto kfn = chain_kernel<T, TM>;
+  const size_t smem = sizeof(T) * ((size_t)2 * P * a.rin_max + (size_t)P * a.n + 2 * BK * P + 2 * BK * (ct_max + 2));
+  auto kfn = ct_max <= 64 ? chain_kernel<T, TM, 64> : chain_kernel<T, TM, sizeof(T) == 8 ? 96 : 128>;
   PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   a.blocks0 = (a.side[0].N + P - 1) / P;
   const int64_t blocks = a.blocks0 + (a.side[1].N + P - 1) / P;
@@ -792,12 +794,13 @@ static pttk_status chain_run(const pttk_tt* tt, const void* X, int64_t N_s, cons
       st.R_out = rout;
       st.coord = coord;
       st.magic = (uint32_t)((0x100000000ull + rin - 1) / rin);
-      // the pass width with the fewest padded columns, the widest of equals
+      // The pass width with the fewest padded columns, the widest of equals; FP64 takes no 128, whose
+      // accumulators would leave room for one block an SM.
       st.ct = 0;
       if (rout > NARROW) {
         st.ct = 64;
         for (int ct : {96, 128})
-          if ((rout + ct - 1) / ct * ct <= (rout + st.ct - 1) / st.ct * st.ct) st.ct = ct;
+          if ((ct == 96 || !fp64) && (rout + ct - 1) / ct * ct <= (rout + st.ct - 1) / st.ct * st.ct) st.ct = ct;
       }
       ct_max = std::max(ct_max, st.ct);
       const int bj = sd == 0 ? coord : tt->d + tt->dtheta + coord;
@@ -818,7 +821,7 @@ static pttk_status chain_run(const pttk_tt* tt, const void* X, int64_t N_s, cons
   int tm = fp64 ? 4 : 8;
   auto smem_of = [&](int t) {
     const size_t P = 16 * (size_t)t;
-    return elem * (2 * P * a.rin_max + P * a.n + 2 * BK * P + 2 * BK * ((size_t)ct_max + 4));
+    return elem * (2 * P * a.rin_max + P * a.n + 2 * BK * P + 2 * BK * ((size_t)ct_max + 2));
   };
   auto blocks_of = [&](int t) { return (N_s + 16 * t - 1) / (16 * t) + (N_t + 16 * t - 1) / (16 * t); };
   while (tm > 1 && (smem_of(tm) > 227 * 1024 || blocks_of(tm) < sm_count())) tm /= 2;
