@@ -348,7 +348,8 @@ __global__ void __launch_bounds__(256) chain_back_step(const T* __restrict__ X, 
 // read as broadcasts; S_2 and gbar_2 (RB values, R_2 padded) in registers; the scalars that the loops
 // index (T_j(x_2), T_j'(x_2), S_1, gbar_1) in shared memory, one column per thread. About
 // 11k FMAs a point at ranks 9, 44: at N = 500k, n = 12 the separate kernels (S_1, S_2, Q and gbar
-// in memory, shared-memory atomics per term) took 16.4 ms.
+// in memory, shared-memory atomics per term) took 16.4 ms, this one 0.525 ms with scalar FP32 FMAs and 0.435 ms
+// with the two-wide ones. What bounds it: issue, and the FP64 pipe for the bases.
 // The bases are formed in FP64 and rounded to T.
 constexpr int AF_THREADS = 128;
 
@@ -384,6 +385,50 @@ size_t adj_smem(int d, int n, int r1, int rb) {
   const size_t shared = (size_t)n * r1 + (size_t)n * (d == 3 ? rb : d == 2 ? r1 : 1) + (d == 3 ? (size_t)r1 * n * rb : 0);
   const size_t per = (size_t)3 * n + 2 * r1;
   return sizeof(T) * ((shared + 3) / 4 * 4 + per * AF_THREADS);
+}
+
+// acc[b] = m x[b] + acc[b], b < B (even), in FP32 by the two-wide instructions: half as many to issue, each half
+// rounding as fmaf does
+template <int B>
+__device__ __forceinline__ void axpy(float m, const float* x, float* acc) {
+  uint64_t mm;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(mm) : "f"(m));
+#pragma unroll
+  for (int b = 0; b < B; b += 2) {
+    uint64_t y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(x[b]), "f"(x[b + 1]));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(acc[b]), "f"(acc[b + 1]));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(z) : "l"(mm), "l"(y));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[b]), "=f"(acc[b + 1]) : "l"(z));
+  }
+}
+template <int B>
+__device__ __forceinline__ void axpy(double m, const double* x, double* acc) {
+#pragma unroll
+  for (int b = 0; b < B; ++b) acc[b] = fma(m, x[b], acc[b]);
+}
+// sum of x[b] y[b], b < B (a multiple of 4), in four partial sums
+template <int B>
+__device__ __forceinline__ float dot4(const float* x, const float* y) {
+  uint64_t e[2] = {0, 0};
+#pragma unroll
+  for (int b = 0; b < B; b += 2) {
+    uint64_t u, v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "f"(x[b]), "f"(x[b + 1]));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(y[b]), "f"(y[b + 1]));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(e[(b >> 1) & 1]) : "l"(u), "l"(v));
+  }
+  float e0, e1, e2, e3;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(e0), "=f"(e1) : "l"(e[0]));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(e2), "=f"(e3) : "l"(e[1]));
+  return (e0 + e1) + (e2 + e3);
+}
+template <int B>
+__device__ __forceinline__ double dot4(const double* x, const double* y) {
+  double e[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int b = 0; b < B; ++b) e[b & 3] = fma(x[b], y[b], e[b & 3]);
+  return (e[0] + e[1]) + (e[2] + e[3]);
 }
 
 template <typename T, int D, int RB>
@@ -448,22 +493,15 @@ __global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, cons
           const T sa = S1[al * AF_THREADS];
           const T* row = G2 + (size_t)al * n * RB;
           for (int j = 0; j < n; ++j, row += RB) {
-            const T m = sa * T2[j * AF_THREADS];
-#pragma unroll
-            for (int b = 0; b < RB; ++b) s2[b] = fma(m, row[b], s2[b]);
+            axpy<RB>(sa * T2[j * AF_THREADS], row, s2);
           }
         }
         T dx3 = T(0);
         cheb_each(x[2], a.lo[2], a.hi[2], n, [&](int j, double t, double dt) {
           const T tj = (T)t * wp;
           const T* row = q + j * RB;
-          T e[4] = {T(0), T(0), T(0), T(0)};
-#pragma unroll
-          for (int b = 0; b < RB; ++b) {
-            gb[b] = fma(tj, row[b], gb[b]);
-            e[b & 3] = fma(s2[b], row[b], e[b & 3]);
-          }
-          dx3 = fma((T)dt, (e[0] + e[1]) + (e[2] + e[3]), dx3);
+          axpy<RB>(tj, row, gb);
+          dx3 = fma((T)dt, dot4<RB>(s2, row), dx3);
         });
         T dx2 = T(0);
         for (int al = 0; al < r1; ++al) {
@@ -471,10 +509,7 @@ __global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, cons
           const T* row = G2 + (size_t)al * n * RB;
           T g1a = T(0), da = T(0);
           for (int j = 0; j < n; ++j, row += RB) {
-            T e[4] = {T(0), T(0), T(0), T(0)};
-#pragma unroll
-            for (int b = 0; b < RB; ++b) e[b & 3] = fma(gb[b], row[b], e[b & 3]);
-            const T qv = (e[0] + e[1]) + (e[2] + e[3]);
+            const T qv = dot4<RB>(gb, row);
             da = fma(D2[j * AF_THREADS], qv, da);
             g1a = fma(T2[j * AF_THREADS], qv, g1a);
           }
