@@ -1081,9 +1081,60 @@ struct SvdPart {
   Buf core;                   // m x r, unit columns in decreasing singular value
 };
 
+// Cuts the parts' kept rows back to where the pivoted QR of all of them together reaches ||R22||^2 <= stop2
+// (see svd_factor); A = R1^T keeps its leading columns.
+static pttk_status cut_parts(std::vector<SvdPart>& parts, double stop2, cudaStream_t s) {
+  const size_t np = parts.size();
+  std::vector<std::vector<double>> diag(np), row(np);  // |R_jj|, ||R[j, :]||
+  std::vector<Buf> norms(np);
+  for (size_t i = 0; i < np; ++i) {
+    SvdPart& pt = parts[i];
+    if (pt.kq == 0) continue;
+    const int64_t q = pt.q();
+    diag[i].resize(pt.kq);
+    row[i].resize(pt.kq);
+    PTTK_TRY(norms[i].alloc(pt.kq, s));
+    colnorm_kernel<<<(unsigned)(((int64_t)pt.kq * 32 + 255) / 256), 256, 0, s>>>(pt.A.p, q, pt.kq, norms[i].p); pttk::count_launch();
+    PTTK_CUDA(cudaMemcpyAsync(row[i].data(), norms[i].p, sizeof(double) * pt.kq, cudaMemcpyDeviceToHost, s));
+    PTTK_CUDA(cudaMemcpy2DAsync(diag[i].data(), sizeof(double), pt.A.p, sizeof(double) * (q + 1), sizeof(double), pt.kq,
+                                cudaMemcpyDeviceToHost, s));
+  }
+  PTTK_CUDA(cudaStreamSynchronize(s));
+  // left[i][j]: the square of part i's block after j steps, summed from its end
+  std::vector<std::vector<double>> left(np);
+  std::vector<int> at(np, 0);
+  for (size_t i = 0; i < np; ++i) {
+    left[i].assign(parts[i].kq + 1, parts[i].tail2);
+    for (int j = parts[i].kq - 1; j >= 0; --j) left[i][j] = left[i][j + 1] + row[i][j] * row[i][j];
+  }
+  while (true) {
+    double sum = 0.0;
+    for (size_t i = 0; i < np; ++i) sum += left[i][at[i]];
+    if (sum <= stop2) break;
+    int next = -1;
+    for (size_t i = 0; i < np; ++i)
+      if (at[i] < parts[i].kq && (next < 0 || fabs(diag[i][at[i]]) > fabs(diag[next][at[next]]))) next = (int)i;
+    if (next < 0) break;
+    ++at[next];
+  }
+  for (size_t i = 0; i < np; ++i) {
+    const int k = std::max(at[i], std::min(1, parts[i].kq));
+    parts[i].kq = k;
+    parts[i].tail2 = left[i][k];
+  }
+  return PTTK_OK;
+}
+
 // Factors the parts: R1^T V = U' Sigma of the kept rows R1 of the pivoted QR (A holds U' Sigma), with the
 // singular values. delta and stop_frac: the pivoted QRs stop once their discarded blocks together have
 // ||R22||_F <= stop_frac delta.
+//
+// Several parts stop where the pivoted QR of the whole unfolding would. That QR takes the part with the
+// largest trailing column at each step and leaves the others alone, so its steps are the parts' own, merged by
+// decreasing |R_jj|. Each part factors until its block is a sixteenth of its share (in squares), and the host cuts
+// the parts back to the step of the merged order at which the blocks together are small enough: the kept rows,
+// and with them the ranks of unfoldings whose tail lies within stop_frac^2 of the threshold, are
+// those of one QR.
 static pttk_status svd_factor(std::vector<SvdPart>& parts, double delta, double stop_frac, StageClock& clk, int k,
                               cudaStream_t s) {
   const int np = (int)parts.size();
@@ -1110,7 +1161,7 @@ static pttk_status svd_factor(std::vector<SvdPart>& parts, double delta, double 
       PTTK_CUDA(cudaMemcpyAsync(pt.qrin.p, pt.X, sizeof(double) * pt.m * pt.c, cudaMemcpyDeviceToDevice, s));
     }
     PTTK_TRY(pt.R.alloc(q * q, s));
-    qr.push_back(Qr{pt.qrin.p, Mqr, (int)q, stop * stop / np, pt.R.p, pt.perm.ints()});
+    qr.push_back(Qr{pt.qrin.p, Mqr, (int)q, np == 1 ? stop * stop : stop * stop / (16.0 * np), pt.R.p, pt.perm.ints()});
   }
   clk.mark(k, "layout");
   PTTK_TRY(householder_batch(qr, s));
@@ -1118,7 +1169,7 @@ static pttk_status svd_factor(std::vector<SvdPart>& parts, double delta, double 
   // one-sided Jacobi on A = R1^T (q x kq), R1 = the kept rows of R in pivoted column order: R1^T V = U'
   // Sigma, so R1 = V Sigma U'^T and the right singular vectors of R1 (= of the pivoted QR input, up to
   // the discarded R22) are the normalised columns of the rotated R1^T; columns below (stop_frac / 30)
-  // delta / sqrt(kq) together carry < (stop_frac / 30)^2 delta^2, and pairs of them are skipped.
+  // delta / sqrt(kq), kq over all parts, together carry < (stop_frac / 30)^2 delta^2, and pairs of them are skipped.
   // Where R1^T has at least 2.5 times as many rows as columns: a second pivoted QR, R1^T P2 = Q2 R2, and
   // the Jacobi on R2 (kq x kq), whose columns have the Gram matrix of R1^T P2's and so take the same
   // rotations, accumulated in V; the rotated R1^T is then R1^T (P2 V), one DGEMM. Each rotation touches
@@ -1137,11 +1188,18 @@ static pttk_status svd_factor(std::vector<SvdPart>& parts, double delta, double 
     pt.kq = qr[i].k;
     pt.tail2 = qr[i].tail2;
     pt.qrin.free();
-    if (clk.on) fprintf(stderr, "pttk: tt-svd step %d kept %d of %lld rows of R, ||R22|| %.3e\n", k + 1, pt.kq, (long long)q, sqrt(pt.tail2));
     PTTK_TRY(pt.A.alloc(q * pt.kq, s));
     gather_rt_kernel<<<grid1d(q * pt.kq, 256), 256, 0, s>>>(pt.R.p, q, pt.kq, pt.perm.ints(), pt.A.p); pttk::count_launch();
+  }
+  if (np > 1) PTTK_TRY(cut_parts(parts, stop * stop, s));
+  double kq_all = 0.0;
+  for (const SvdPart& pt : parts) kq_all += pt.kq;
+  const double skip = (stop_frac / 30.0) * delta / sqrt(kq_all);
+  for (SvdPart& pt : parts) {
+    const int64_t q = pt.q();
+    if (clk.on) fprintf(stderr, "pttk: tt-svd step %d kept %d of %lld rows of R, ||R22|| %.3e\n", k + 1, pt.kq, (long long)q, sqrt(pt.tail2));
     if (2 * q >= 5 * (int64_t)pt.kq && pt.kq >= 2) second.push_back(Second{&pt});
-    else jac.push_back(Jac{pt.A.p, q, pt.kq, (stop_frac / 30.0) * delta / sqrt((double)pt.kq)});
+    else jac.push_back(Jac{pt.A.p, q, pt.kq, skip});
   }
   for (Second& sc : second) {
     const int64_t q = sc.pt->q(), kq = sc.pt->kq;
@@ -1160,7 +1218,7 @@ static pttk_status svd_factor(std::vector<SvdPart>& parts, double delta, double 
     PTTK_TRY(sc.V.alloc(kq * kq, s));
     PTTK_TRY(sc.PV.alloc(kq * kq, s));
     eye_kernel<<<grid1d(kq * kq, 256), 256, 0, s>>>(sc.V.p, kq); pttk::count_launch();
-    jac.push_back(Jac{sc.Rd.p, k2, (int)kq, (stop_frac / 30.0) * delta / sqrt((double)kq), sc.V.p, kq});
+    jac.push_back(Jac{sc.Rd.p, k2, (int)kq, skip, sc.V.p, kq});
   }
   PTTK_TRY(jacobi_batch(jac, s));
   for (Second& sc : second) {
@@ -1478,6 +1536,13 @@ pttk_status tt_svd_run(pttk_tt* tt, double* X, double tol, cudaStream_t s) {
     }
     std::vector<int> order;
     const int r = truncation(sigma, delta, order, tail2);
+    if (clk.on) {
+      double t = tail2;
+      for (int i = (int)sigma.size() - 1; i >= r; --i) t += sigma[order[i]] * sigma[order[i]];
+      const double sr = sigma[order[r - 1]];
+      fprintf(stderr, "pttk: tt-svd step %d rank %d: tail^2 / delta^2 at r %.6f, at r - 1 %.6f, ||R22||^2 %.6f\n", k + 1, r, t / (delta * delta),
+              (t + sr * sr) / (delta * delta), tail2 / (delta * delta));
+    }
     std::vector<std::vector<int>> ids(parts.size());
     std::vector<unsigned> qn(r);
     for (int a = 0; a < r; ++a) {
