@@ -286,9 +286,9 @@ bool kv_symmetric(int64_t N, bool fp32) {
   return !fp32 && S <= 24576;
 }
 
-// doubles of scratch for one product
-size_t kv_part_elems(int64_t N, bool fp32) {
-  if (!kv_symmetric(N, fp32)) return (size_t)kv_splits(N) * N;
+// doubles of scratch for one product (sym: the symmetric form)
+size_t kv_part_elems(int64_t N, bool sym) {
+  if (!sym) return (size_t)kv_splits(N) * N;
   int T, S, nS;
   kv_sym_shape(N, &T, &S, &nS);
   return (size_t)nS * N;
@@ -307,12 +307,12 @@ pttk_status kv_sym_launch(int kind, const double* X, int64_t N, const KvArgs& k,
   return PTTK_OK;
 }
 
-// out = (K + s2 I) v; part: scratch of kv_part_elems(N, fp32) doubles
+// out = (K + s2 I) v; part: scratch of kv_part_elems(N, sym) doubles
 pttk_status kv_launch(int kind, int d, const double* X, int64_t N, double l, double s2, const double* v, double* out,
-                      bool fp32, double* part, cudaStream_t s) {
+                      bool fp32, bool sym, double* part, cudaStream_t s) {
   PTTK_PROF("gp_kv", s);
   int ncs;
-  if (!kv_symmetric(N, fp32)) {
+  if (!sym) {
     ncs = kv_splits(N);
     const int64_t cols = ((N + ncs - 1) / ncs + GTILE - 1) / GTILE * GTILE;
     const dim3 grid((unsigned)((N + GT - 1) / GT), (unsigned)ncs);
@@ -380,8 +380,13 @@ pttk_status pttk_gp_kv(int kernel, int d, const double* X, int64_t N, const doub
   if (prec != PTTK_FP64 && prec != PTTK_FP32) return set_error(PTTK_EINVAL, "K v: prec must be PTTK_FP64 or PTTK_FP32");
   cudaStream_t s = as_stream(stream);
   double* part = nullptr;
-  PTTK_CUDA(ws_malloc(&part, sizeof(double) * kv_part_elems(N, prec == PTTK_FP32), s));
-  const pttk_status st = kv_launch(kernel, d, X, N, theta[0], s2, v, out, prec == PTTK_FP32, part, s);
+  bool sym = kv_symmetric(N, prec == PTTK_FP32);
+  if (sym && ws_malloc(&part, sizeof(double) * kv_part_elems(N, true), s) != cudaSuccess) {
+    cudaGetLastError();  // the general form needs less scratch
+    sym = false;
+  }
+  if (!sym) PTTK_CUDA(ws_malloc(&part, sizeof(double) * kv_part_elems(N, false), s));
+  const pttk_status st = kv_launch(kernel, d, X, N, theta[0], s2, v, out, prec == PTTK_FP32, sym, part, s);
   cudaFreeAsync(part, s);
   return st;
 }
@@ -407,7 +412,13 @@ pttk_status pttk_gp_pcg(int kernel, int d, const double* X, int64_t N, const dou
   PTTK_TRY(sc.get(&Ap, N));
   PTTK_TRY(sc.get(&part, nparts));
   double* kvpart = nullptr;
-  PTTK_TRY(sc.get(&kvpart, kv_part_elems(N, prec == PTTK_FP32)));
+  bool sym = kv_symmetric(N, prec == PTTK_FP32);
+  if (sym && sc.get(&kvpart, kv_part_elems(N, true)) != PTTK_OK) {
+    cudaGetLastError();
+    clear_error();
+    sym = false;
+  }
+  if (!sym) PTTK_TRY(sc.get(&kvpart, kv_part_elems(N, false)));
   if (m > 0) {
     PTTK_TRY(sc.get(&coef, m));
     PTTK_TRY(sc.get(&gpart, (size_t)gparts * m));
@@ -436,7 +447,7 @@ pttk_status pttk_gp_pcg(int kernel, int d, const double* X, int64_t N, const dou
   double rn = bn;
   int it = 0;
   while (rn > tol * bn && it < maxit) {
-    PTTK_TRY(kv_launch(kernel, d, X, N, l, s2, p, Ap, prec == PTTK_FP32, kvpart, s));
+    PTTK_TRY(kv_launch(kernel, d, X, N, l, s2, p, Ap, prec == PTTK_FP32, sym, kvpart, s));
     double pAp = 0.0;
     PTTK_TRY(dot_host(p, Ap, N, part, nparts, &pAp, s));
     if (!(pAp > 0.0)) return set_error(PTTK_EDOMAIN, "CG: p^T A p <= 0 (the matrix is not positive definite)");

@@ -401,8 +401,25 @@ __global__ void __launch_bounds__(256) expand_kernel(GridArgs a, const T* __rest
   }
 }
 
+// Extents of the modes (a source mode is folded where the boxes have the same centre, see the file comment)
+// and the leading block of m1 modes held in shared memory.
+void plan_tiles(GridArgs& a, bool fold, size_t elem) {
+  const size_t budget = elem == 8 ? 170000 : 90000;
+  for (int j = 0; j < a.D; ++j) a.ext[j] = a.n;
+  for (int j = 0; fold && j < a.d; ++j)
+    if (a.lo[j] + a.hi[j] == a.lo[a.d + a.dtheta + j] + a.hi[a.d + a.dtheta + j]) a.ext[j] = (a.n + 1) / 2;
+  a.m1 = 1;
+  a.tile = a.ext[0];
+  while (a.m1 < a.D && (size_t)(a.tile * a.ext[a.m1]) * elem <= budget) {
+    a.tile *= a.ext[a.m1];
+    ++a.m1;
+  }
+  a.ntiles = 1;
+  for (int j = a.m1; j < a.D; ++j) a.ntiles *= a.ext[j];
+}
+
 template <typename T, int NB>
-pttk_status launch_all(const GridArgs& a, T* C, cudaStream_t st) {
+pttk_status launch_all(GridArgs a, T* C, cudaStream_t st) {
   // folded tensor: in workspace memory, expanded into C at the end
   int64_t total = 1, folded = 1, tin = 1, tout = 1;
   for (int j = 0; j < a.D; ++j) {
@@ -422,8 +439,17 @@ pttk_status launch_all(const GridArgs& a, T* C, cudaStream_t st) {
   } fold{nullptr, st};
   T* F = C;
   if (folded != total) {
-    PTTK_CUDA(ws_malloc(&fold.p, sizeof(T) * (size_t)folded, st));
-    F = fold.p;
+    const cudaError_t e = ws_malloc(&fold.p, sizeof(T) * (size_t)folded, st);
+    if (e == cudaSuccess) {
+      F = fold.p;
+    } else if (e == cudaErrorMemoryAllocation) {  // no room beside C: the whole grid in place
+      cudaGetLastError();
+      fold.p = nullptr;
+      plan_tiles(a, false, sizeof(T));
+      folded = total;
+    } else {
+      PTTK_CUDA(e);
+    }
   }
   const int threads = sizeof(T) == 8 ? 512 : 256;
   const size_t smem = sizeof(T) * (a.tile + (size_t)a.D * a.n + 2 * (NB / 2) * (NB / 2) + 2 * a.n + FEXP_N +
@@ -556,21 +582,7 @@ pttk_status grid_coeffs_launch(int kernel, int d, int dtheta, int n, const doubl
     a.lo[j] = box[j][0];
     a.hi[j] = box[j][1];
   }
-  // leading block of m1 modes held in shared memory
-  const size_t elem = fp64 ? 8 : 4;
-  const size_t budget = fp64 ? 170000 : 90000;
-  // a source mode is folded where the boxes have the same centre (see the file comment)
-  for (int j = 0; j < a.D; ++j) a.ext[j] = n;
-  for (int j = 0; j < d; ++j)
-    if (a.lo[j] + a.hi[j] == a.lo[d + dtheta + j] + a.hi[d + dtheta + j]) a.ext[j] = (n + 1) / 2;
-  a.m1 = 1;
-  a.tile = a.ext[0];
-  while (a.m1 < a.D && (size_t)(a.tile * a.ext[a.m1]) * elem <= budget) {
-    a.tile *= a.ext[a.m1];
-    ++a.m1;
-  }
-  a.ntiles = 1;
-  for (int j = a.m1; j < a.D; ++j) a.ntiles *= a.ext[j];
+  plan_tiles(a, true, fp64 ? 8 : 4);
   // the per-nu tables live until the kernels that read them have run: released stream-ordered
   // on every return path
   struct Tables {
