@@ -169,9 +169,9 @@ def kernel_rooflines(prof, steps, ranks, d, dtheta, n, N, hbm, dfma):
     TFLOP/s):
     - apply, domain, mode_transform: HBM bytes (FP32 factors; FP32 points; one FP64 and one
       FP32 grid, each with its D - m1 = 4 strided passes that read and write every entry);
-    - dgemm: FP64 flops of the TT-SVD's projections X <- G_k^T X alone, so its fraction is a
-      lower bound (the tall steps' X V products and the preconditioned Jacobi's R1^T (P2 V)
-      are not counted);
+    - dgemm: FP64 flops of the TT-SVD's projections X <- G_k^T X alone, on the whole unfoldings
+      (the tall steps' X V products and the preconditioned Jacobi's R1^T (P2 V) are not counted;
+      parity sectors execute about a tenth of what is counted);
     - householder, jacobi, theta_core: null, with the reason (their work depends on the QR's
       stopping step, the Jacobi's sweeps, or is latency-bound)."""
     D = 2 * d + dtheta
@@ -199,7 +199,8 @@ def kernel_rooflines(prof, steps, ranks, d, dtheta, n, N, hbm, dfma):
     hbm_entry("domain", m_cnt * 4.0 * 2 * N * d, "reads X and Y once (N x d each, FP32)")
     t_ms, t_cnt = ms_of("mode_transform")
     hbm_entry("mode_transform", steps * 4 * (16.0 + 8.0) * total,
-              "per step 4 passes over the FP64 grid (16 B per entry) and 4 over the FP32 grid (8 B)")
+              "per step 4 passes over the FP64 grid (16 B per entry) and 4 over the FP32 grid (8 B), counted on the "
+              "whole grid: the reflection-folded one that is transformed has a quarter of its entries at d = 3")
     g_ms, g_cnt = ms_of("dgemm")
     if g_cnt and g_ms > 0:
         proj = 0.0
@@ -210,7 +211,8 @@ def kernel_rooflines(prof, steps, ranks, d, dtheta, n, N, hbm, dfma):
         ach = steps * proj / (g_ms / 1000.0) / 1e12
         out["dgemm"] = {"bound": "alu (FP64 FMA)", "achieved": ach, "peak": dfma, "unit": "TFLOP/s",
                         "frac_lower_bound": ach / dfma, "launches": g_cnt,
-                        "note": "the TT-SVD projections' flops only: a lower bound of the DGEMM work"}
+                        "note": "the TT-SVD projections' flops on the whole unfoldings, nothing else; where parity sectors are "
+                                "found (d = 3: a tenth of these flops is executed) the fraction passes 1"}
     for name, why in (("householder", "work depends on the step at which each pivoted QR stops"),
                       ("jacobi", "work depends on the number of sweeps"),
                       ("theta_core", "latency-bound: a few small contractions per theta")):
@@ -453,8 +455,7 @@ def main():
     roof_dominant = {"kernel": dom[0], "ms_total": dom[1][0], "launches": dom[1][1],
                      "share_of_timed_kernel_time": dom[1][0] / max(prof_total, 1e-9),
                      "bound": "alu (FP64)" if dom[0] in ("jacobi", "householder", "dgemm", "grid_tile") else "tensor",
-                     "note": "the FP64 offline stage (grid, pivoted QR, Jacobi) holds most of the step; see kernel_ms "
-                             "and roofline_grid_fp64"}
+                     "note": "largest share of the step's kernel time; see kernel_ms"}
     g32_bytes = total * 4.0 * args.steps * world
     roof_grid = {"fp64_entries_per_s": total * args.steps * world / (g64_ms / 1000.0),
                  "fp32_entries_per_s": total * args.steps * world / (g32_ms / 1000.0),
@@ -843,8 +844,9 @@ def run_extras(torch, P, W, w, tt, X32, Y32, wv, thetas, state, flush, ev, pk, h
                       "roofline": {"bound": "alu (FP32 FMA)", "achieved": adj_flops / (adj_ms / 1000.0) / 1e12,
                                    "peak": pk["ffma"], "unit": "TFLOP/s",
                                    "frac": adj_flops / (adj_ms / 1000.0) / 1e12 / pk["ffma"],
-                                   "note": "reverse pass for dL/dX (FP32 SIMT: recomputed chain prefix and two "
-                                           "reverse products per step), counted as 3x the source chain's flops"}}
+                                   "note": "reverse pass for dL/dX (FP32 SIMT), counted as 3x the source chain's flops; "
+                                           "its last step needs a vector only, so the executed flops are a tenth of it "
+                                           "and the fraction passes 1"}}
 
     # TT-Round (Algorithm 1) of the d = 3 TT: to looser tolerances, and of its sum with itself
     # (ranks doubled), back to 1e-10
