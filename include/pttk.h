@@ -441,8 +441,7 @@ void pttk_batch_free(pttk_batch* b);
  * accumulators or staging tiles do not fit fall back to configuration 1); 1 and 2: the latter without
  * the epilogue warps, with 128- or 64-byte chunks of K per row; 3, 4, 5: for the FP16/BF16
  * forms, the kernel that generates A in tensor memory and keeps the chain's intermediate in
- * registers, run in thread-block clusters of 1, 2 or 4 CTAs that share each core chunk by a
- * multicast copy (ranks it cannot hold fall back to configuration 1); 6: for the FP16/BF16
+ * registers (4 and 5 launch what 3 launches; ranks it cannot hold fall back to configuration 1); 6: for the FP16/BF16
  * forms, A in tensor memory with separate epilogue warps and a B ring of 3-4 slots in the
  * shared memory A no longer takes (ranks it cannot hold fall back to the kernel with A in shared
  * memory); 7: A in shared memory with epilogue warps, 64-byte chunks of K per row in a ring of 4

@@ -1012,8 +1012,8 @@ struct TsArgs {
   int s0_coord[2];
   float s0_lo[2], s0_hi[2];
   int64_t N[2];
-  int64_t T0p;       // source tiles, padded to a multiple of the cluster size
-  int64_t nitems;    // cluster items: CL consecutive tiles of one side each
+  int64_t T0p;       // source tiles
+  int64_t nitems;    // tiles of both sides
   const float* pts[2];
   float* out[2];
   int* status;
@@ -1027,40 +1027,16 @@ struct TsArgs {
   uint32_t b_slot_bytes;  // bytes reserved per B part per slot
 };
 
-// bulk copy of `bytes` from global memory to the same shared-memory offset in every CTA of the
-// cluster named by `mask`, each destination's mbarrier (same offset) receiving the bytes
-__device__ __forceinline__ void tma_load_1d_mc(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "h"(mask)
-      : "memory");
-}
-// arrive on the mbarrier at this offset in every CTA of `mask` once this thread's MMAs complete
-__device__ __forceinline__ void umma_commit_mc(uint64_t* bar, uint16_t mask) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-                   smem_u32(bar)),
-               "h"(mask)
-               : "memory");
-}
-
 // Warp roles as in chain_tc_kernel: warp 0 (one lane) streams core chunks into the NS-deep
 // shared-memory ring with TMA, warp 1 (one lane) issues the MMAs, warps 2..17 generate A into
 // the NS-deep TMEM ring and run the epilogues.
 //
-// Every 128-point tile streams the whole oriented core through shared memory, so at these
-// ranks the core traffic from L2 rivals the MMA time. The CL CTAs of a thread-block cluster
-// therefore work in lockstep on CL consecutive tiles of one side (a cluster item; each side's
-// tile count is padded to a multiple of CL with empty tiles), and each CTA loads 1/CL of every
-// core chunk with a multicast copy into all CL CTAs: the L2 traffic of the cores falls by CL.
 // Barriers per slot: full_a (16 generator warps arrive after their tcgen05.st completed),
-// full_b (the chunk's bytes from all CL copies), empty_a (the local MMAs of the slot completed:
-// the TMEM slot may be rewritten), empty_b (the MMAs of the slot completed in every CTA of the
-// cluster: the shared-memory slot, written by every CTA's copies, may be reloaded).
-template <int FMT, bool SPLIT, int NS, int CL>
+// full_b (the chunk's bytes), empty_a (the MMAs of the slot completed: the TMEM slot may be
+// rewritten), empty_b (the same MMAs: the shared-memory slot may be reloaded).
+template <int FMT, bool SPLIT, int NS>
 __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
   constexpr int PARTS = SPLIT ? 2 : 1;
-  constexpr uint16_t MASK = (uint16_t)((1u << CL) - 1u);
   extern __shared__ __align__(1024) uint8_t smem[];
   const int bv_ld = a.bv_ld;
   uint8_t* b_base = smem;                                                // NS x PARTS x b_slot_bytes
@@ -1079,14 +1055,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int crank = CL > 1 ? (int)cluster_rank() : 0;
-  const int64_t cid = blockIdx.x / CL, ncl = gridDim.x / CL;
+  const int64_t cid = blockIdx.x, ncl = gridDim.x;
   if (tid == 0) {
     for (int i = 0; i < NS; ++i) {
       mbar_init(&full_a[i], NGEN_WARPS);
       mbar_init(&full_b[i], 1);
       mbar_init(&empty_a[i], 1);
-      mbar_init(&empty_b[i], CL);
+      mbar_init(&empty_b[i], 1);
     }
     mbar_init(&acc_ready[0], 1);
     mbar_init(&acc_ready[1], 1);
@@ -1101,19 +1076,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (CL > 1) cluster_sync_all();  // every CTA's barriers exist before any copy or commit reaches them
   const uint32_t tmem = *tmem_slot;
   const int64_t nitems = a.nitems;
   const int nsteps = a.nsteps;
-  // side, first row and row count of this CTA's tile in cluster item k
-  auto item_side = [&](int64_t k) -> int { return k * CL < a.T0p ? 0 : 1; };
-  auto item_row0 = [&](int64_t k) -> int64_t {
-    const int sd = item_side(k);
-    return (k * CL + crank - (sd ? a.T0p : 0)) * TILE_M;
-  };
+  // side and first row of tile k
+  auto item_side = [&](int64_t k) -> int { return k < a.T0p ? 0 : 1; };
+  auto item_row0 = [&](int64_t k) -> int64_t { return (k - (item_side(k) ? a.T0p : 0)) * TILE_M; };
 
   if (warp == 0) {
-    // ---------------- TMA producer: this CTA's share of every chunk, to every CTA ----------------
+    // ---------------- TMA producer ----------------
     if (lane == 0) {
       uint32_t h = 0;
       bool ok = true;
@@ -1122,24 +1093,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
         for (int si = 0; si < nsteps && ok; ++si) {
           const TsStepS& st = steps[sd * 3 + si];
           const uint32_t bytes = st.bytes;
-          // the chunk's 8-row groups are split over the CL CTAs (the last ones may get none)
-          const uint32_t groups = bytes / st.sbo, gper = (groups + CL - 1) / CL;
-          const uint32_t off = min((uint32_t)crank * gper, groups) * st.sbo;
-          const uint32_t len = min(gper * st.sbo, bytes - off);
           for (int c = 0; c < st.nchunks; ++c, ++h) {
             const uint32_t slot = h % NS;
             if (h >= NS && !mbar_wait(&empty_b[slot], ((h / NS) - 1) & 1, abort_flag)) { ok = false; break; }
             uint8_t* bh = b_base + (size_t)slot * PARTS * a.b_slot_bytes;
             mbar_arrive_expect_tx(&full_b[slot], SPLIT ? 2 * bytes : bytes);
-            if (len > 0) {
-              if (CL > 1) {
-                tma_load_1d_mc(bh + off, st.hi + (size_t)c * bytes + off, len, &full_b[slot], MASK);
-                if (SPLIT) tma_load_1d_mc(bh + a.b_slot_bytes + off, st.lo + (size_t)c * bytes + off, len, &full_b[slot], MASK);
-              } else {
-                tma_load_1d(bh, st.hi + (size_t)c * bytes, bytes, &full_b[slot]);
-                if (SPLIT) tma_load_1d(bh + a.b_slot_bytes, st.lo + (size_t)c * bytes, bytes, &full_b[slot]);
-              }
-            }
+            tma_load_1d(bh, st.hi + (size_t)c * bytes, bytes, &full_b[slot]);
+            if (SPLIT) tma_load_1d(bh + a.b_slot_bytes, st.lo + (size_t)c * bytes, bytes, &full_b[slot]);
           }
         }
       }
@@ -1187,8 +1147,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
               }
             }
             umma_commit(&empty_a[slot]);
-            if (CL > 1) umma_commit_mc(&empty_b[slot], MASK);
-            else umma_commit(&empty_b[slot]);
+            umma_commit(&empty_b[slot]);
             if (c == nch - 1) umma_commit(&acc_ready[ab]);
           }
         }
@@ -1410,8 +1369,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) chain_ts_kernel(TsArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // no CTA leaves while a peer may still copy into its shared memory or commit to its barriers
-  if (CL > 1) cluster_sync_all();
   if (warp == 1) tmem_dealloc(tmem, (uint32_t)a.tmem_cols);
 }
 
@@ -2024,8 +1981,8 @@ static pttk_status build_images(const pttk_tt* tt, const TcImageCache* cache, pt
 // with d >= 2 whose ranks fit it, else the shared-memory kernel with dedicated epilogue warps and
 // double-buffered accumulators (chain_tce_kernel), 128 bytes of K per chunk row;
 // 1 and 2: the shared-memory kernel without them, with {KCB, NSLOT} below; 3..5: the TS kernel
-// (A in tensor memory, a ring of 3 slots) in thread-block clusters of 1, 2 or 4 CTAs, for the
-// kind::f16 forms whose ranks fit it. A configuration whose kernel cannot hold the ranks falls
+// (A in tensor memory, a ring of 3 slots), for the kind::f16 forms whose ranks fit it (4 and 5 are
+// the same launch as 3, for callers that name them). A configuration whose kernel cannot hold the ranks falls
 // back to configuration 1. 6: A in tensor memory with the epilogue warps (falls back to 0).
 // 7: configuration 0 with 64 bytes of K per chunk row and a ring of 4 slots: the same shared
 // memory as 0's 128-byte ring of 2 at large ranks, so each core chunk's copy has three chunks
@@ -2035,12 +1992,10 @@ static const int kTcConfigsSplit[2][2] = {{128, 2}, {64, 4}};
 constexpr int kTceConfigs = 1, kTcSubConfigs = 2, kTsConfigs = 3, kTseConfigs = 1, kTce64Configs = 1;
 constexpr int kTceFirst = 0, kSubFirst = kTceFirst + kTceConfigs, kTsFirst = kSubFirst + kTcSubConfigs,
               kTseFirst = kTsFirst + kTsConfigs, kTce64First = kTseFirst + kTseConfigs;
-static const int kTsCluster[kTsConfigs] = {1, 2, 4};
 
 int tc_config_count() { return kTseConfigs + kTceConfigs + kTcSubConfigs + kTsConfigs + kTce64Configs; }
 static bool ts_form(pttk_prec p) { return p == PTTK_FP16 || p == PTTK_FP16X3 || p == PTTK_BF16 || p == PTTK_BF16X3; }
 static bool ts_config(int cfg) { return cfg >= kTsFirst && cfg < kTsFirst + kTsConfigs; }
-static int ts_cluster(int cfg) { return kTsCluster[cfg - kTsFirst]; }
 static bool tse_config(int cfg) { return cfg >= kTseFirst && cfg < kTseFirst + kTseConfigs; }
 static bool tce_config(int cfg) {
   return (cfg >= kTceFirst && cfg < kTceFirst + kTceConfigs) || (cfg >= kTce64First && cfg < kTce64First + kTce64Configs);
@@ -2176,39 +2131,16 @@ static bool ts_plan(const pttk_tt* tt, const TcImageCache* cache, const Images& 
   return true;
 }
 
-// Grid of the TS kernel: one CTA per SM in clusters of CL, as many clusters as can be
-// resident at once (clusters are placed within a GPC, so with CL > 1 a few SMs may stay idle),
-// and no more than there are cluster items.
-template <int FMT, bool SPLIT, int NS, int CL>
+template <int FMT, bool SPLIT, int NS>
 static pttk_status launch_ts(TsArgs a, int64_t T0, int64_t T1, size_t smem, cudaStream_t s) {
-  auto kfn = chain_ts_kernel<FMT, SPLIT, NS, CL>;
+  auto kfn = chain_ts_kernel<FMT, SPLIT, NS>;
   PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  if (CL > 1) PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeNonPortableClusterSizeAllowed, 0));
-  a.T0p = (T0 + CL - 1) / CL * CL;
-  a.nitems = (a.T0p + (T1 + CL - 1) / CL * CL) / CL;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  cfg.blockDim = dim3(TC_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  int64_t nclusters = sm_count() / CL;
-  if (CL > 1) {
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3((unsigned)(nclusters * CL));
-    int active = 0;
-    PTTK_CUDA(cudaOccupancyMaxActiveClusters(&active, kfn, &cfg));
-    if (active < 1) return set_error(PTTK_ENOTSUP, "tensor-core chain: no cluster of this size fits");
-    nclusters = std::min<int64_t>(nclusters, active);
-  }
-  nclusters = std::max<int64_t>(1, std::min<int64_t>(nclusters, a.nitems));
-  cfg.gridDim = dim3((unsigned)(nclusters * CL));
-  PTTK_CUDA(cudaLaunchKernelEx(&cfg, kfn, a));
+  a.T0p = T0;
+  a.nitems = T0 + T1;
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(a.nitems, sm_count()));
+  kfn<<<grid, TC_THREADS, smem, s>>>(a);
   pttk::count_launch();
+  PTTK_CUDA(cudaGetLastError());
   return PTTK_OK;
 }
 
@@ -2338,7 +2270,7 @@ pttk_status factor_build_tc(const pttk_tt* tt, TcImageCache* cache, const float*
     }
   }
   if (ts_config(cfg) && ts_form(prec)) {
-    const int NS = 3, CL = ts_cluster(cfg);
+    const int NS = 3;
     TsArgs a;
     size_t smem = 0;
     if (ts_plan(tt, cache, cache->ts[fi], prec, NS, a, &smem)) {
@@ -2353,16 +2285,9 @@ pttk_status factor_build_tc(const pttk_tt* tt, TcImageCache* cache, const float*
       PTTK_PROF("chain_tc", s);
       const int fmt = form_fmt(prec);
       const bool split = form_split(prec);
-#define PTTK_TS_LAUNCH(F, SP)                                                            \
-  return CL == 4 ? launch_ts<F, SP, 3, 4>(a, T0, T1, smem, s)                            \
-                 : CL == 2 ? launch_ts<F, SP, 3, 2>(a, T0, T1, smem, s) : launch_ts<F, SP, 3, 1>(a, T0, T1, smem, s);
-      if (fmt == FMT_BF16) {
-        if (split) { PTTK_TS_LAUNCH(FMT_BF16, true) }
-        PTTK_TS_LAUNCH(FMT_BF16, false)
-      }
-      if (split) { PTTK_TS_LAUNCH(FMT_FP16, true) }
-      PTTK_TS_LAUNCH(FMT_FP16, false)
-#undef PTTK_TS_LAUNCH
+      if (fmt == FMT_BF16)
+        return split ? launch_ts<FMT_BF16, true, 3>(a, T0, T1, smem, s) : launch_ts<FMT_BF16, false, 3>(a, T0, T1, smem, s);
+      return split ? launch_ts<FMT_FP16, true, 3>(a, T0, T1, smem, s) : launch_ts<FMT_FP16, false, 3>(a, T0, T1, smem, s);
     }
   }
   int KCB, NS;
