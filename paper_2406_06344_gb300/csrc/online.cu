@@ -334,17 +334,54 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && CTMAX == 64 ? 3 : 2) ch
 }
 
 // ---------------- apply: out = U (M (V^T w)) ----------------------------------------
-// partial[b, c] = sum over block b's rows r of V[r, c] w[r], V read as a flat array of 16-byte units (of
-// VW elements, whatever rt is): a unit of P rows (P rt a multiple of VW) always covers the same columns, so thread t
-// keeps VW accumulators, whose column and row offset never change, and takes unit t of every group of P rows;
-// nt = P rt / VW threads make a group, and as many groups as fit run side by side, UNR of them in flight per thread.
-// The accumulators of a column meet in shared memory in a fixed order. (V not 16-byte aligned: VW = 1, P = 1.)
-// What bounds it: the read of V (2.6 TB/s from L2 at this size). 100k x 180 FP32: 34 -> 28 us; 100k x 63 FP64, where a
-// unit holds two columns: 19 -> 22 us, beside a 10 ms chain.
+// partial[b, c] = sum over block b's rows r of V[r, c] w[r], in one of two forms (apply_typed chooses).
+//
+// By columns: threads are 4 row lanes x 64 columns, four rows of loads in flight each.
+template <typename T>
+__global__ void __launch_bounds__(256) vtw_columns_kernel(const T* __restrict__ V, int64_t N, int rt,
+                                                          const T* __restrict__ w, T* __restrict__ partial) {
+  __shared__ T red[4][64];
+  const int64_t per = (N + gridDim.x - 1) / gridDim.x;
+  const int64_t r0 = (int64_t)blockIdx.x * per, r1 = std::min<int64_t>(N, r0 + per);
+  const int cl = threadIdx.x & 63, rl = threadIdx.x >> 6;
+  for (int cb = 0; cb < rt; cb += 64) {
+    const int c = cb + cl;
+    const bool on = c < rt;
+    T acc[1] = {T(0)};
+    int64_t r = r0 + rl;
+    for (; r + 12 < r1; r += 16) {
+      T v[4][1];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const T* src = V + (r + 4 * u) * rt + c;
+        v[u][0] = on ? *src : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const T wr = w[r + 4 * u];
+        acc[0] = fma(v[u][0], wr, acc[0]);
+      }
+    }
+    for (; r < r1; r += 4) {
+      const T wr = w[r];
+      acc[0] = fma(on ? V[r * rt + c] : T(0), wr, acc[0]);
+    }
+    red[rl][cl] = acc[0];
+    __syncthreads();
+    for (int q = threadIdx.x; q < 64; q += blockDim.x)
+      if (cb + q < rt) partial[(int64_t)blockIdx.x * rt + cb + q] = (red[0][q] + red[1][q]) + (red[2][q] + red[3][q]);
+    __syncthreads();
+  }
+}
+
+// Flat: V as an array of 16-byte units (of VW elements, whatever rt is): a unit of P rows (P rt a multiple of VW)
+// always covers the same columns, so thread t keeps accumulators whose columns and row offsets never change (VW for
+// each of the UNR groups in flight, so that no sum is a longer chain than in the form above), and takes unit t of
+// every group of P rows; nt = P rt / VW threads make a group, and as many groups as fit run side by side. The
+// accumulators of a column meet in shared memory in a fixed order.
 template <typename T, int VW>
-__global__ void __launch_bounds__(256) vtw_partial_kernel(const T* __restrict__ V, int64_t N,
-                                                          int rt, int P, const T* __restrict__ w,
-                                                          T* __restrict__ partial) {
+__global__ void __launch_bounds__(256) vtw_flat_kernel(const T* __restrict__ V, int64_t N, int rt, int P,
+                                                       const T* __restrict__ w, T* __restrict__ partial) {
   constexpr int UNR = 4;
   __shared__ T red[256 * VW];
   const int nt = P * rt / VW;
@@ -356,11 +393,12 @@ __global__ void __launch_bounds__(256) vtw_partial_kernel(const T* __restrict__ 
     const int t = tb + threadIdx.x % width, gl = threadIdx.x / width;
     const bool on = gl < lanes;
     int off[VW];
-    T acc[VW];
+    T acc[UNR][VW];
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
       off[e] = (VW * t + e) / rt;
-      acc[e] = T(0);
+#pragma unroll
+      for (int u = 0; u < UNR; ++u) acc[u][e] = T(0);
     }
     auto load = [&](int64_t g, T* v) {
       const T* src = V + g * P * rt + (int64_t)VW * t;
@@ -385,38 +423,71 @@ __global__ void __launch_bounds__(256) vtw_partial_kernel(const T* __restrict__ 
 #pragma unroll
         for (int u = 0; u < UNR; ++u)
 #pragma unroll
-          for (int e = 0; e < VW; ++e) acc[e] = fma(v[u][e], w[(g + u * lanes) * P + off[e]], acc[e]);
+          for (int e = 0; e < VW; ++e) acc[u][e] = fma(v[u][e], w[(g + u * lanes) * P + off[e]], acc[u][e]);
       }
       for (; g < gfull; g += lanes) {
         T v[VW];
         load(g, v);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) acc[e] = fma(v[e], w[g * P + off[e]], acc[e]);
+        for (int e = 0; e < VW; ++e) acc[0][e] = fma(v[e], w[g * P + off[e]], acc[0][e]);
       }
       if (g < g1)
 #pragma unroll
         for (int e = 0; e < VW; ++e) {
           const int64_t row = g * P + off[e];
-          if (row < N) acc[e] = fma(V[g * P * rt + (int64_t)VW * t + e], w[row], acc[e]);
+          if (row < N) acc[0][e] = fma(V[g * P * rt + (int64_t)VW * t + e], w[row], acc[0][e]);
         }
     }
     __syncthreads();
 #pragma unroll
-    for (int e = 0; e < VW; ++e) red[threadIdx.x * VW + e] = acc[e];
+    for (int e = 0; e < VW; ++e) red[threadIdx.x * VW + e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
     __syncthreads();
-    // element VW t + e of a group is column (VW t + e) mod rt; red holds elements VW tb .. of every lane
+    // the lanes' sums, halved until few are left (few columns have up to 256 lanes)
+    int left = lanes;
+    while (left > 16) {
+      const int half = (left + 1) / 2;
+      if (gl + half < left)
+#pragma unroll
+        for (int e = 0; e < VW; ++e) red[threadIdx.x * VW + e] += red[(threadIdx.x + half * width) * VW + e];
+      left = half;
+      __syncthreads();
+    }
+    // element VW t + e of a group is column (VW t + e) mod rt; red holds elements VW tb ..
     for (int c = threadIdx.x; c < rt; c += 256) {
       T sum = T(0);
       for (int el = c; el < P * rt; el += rt) {
         const int q = el - VW * tb;
         if (q < 0 || q >= VW * width) continue;
-        for (int l = 0; l < lanes; ++l) sum += red[(l * width) * VW + q];
+        for (int l = 0; l < left; ++l) sum += red[l * width * VW + q];
       }
       T* dst = partial + (int64_t)blockIdx.x * rt + c;
       *dst = tb == 0 ? sum : *dst + sum;
     }
     __syncthreads();
   }
+}
+
+// The form of V^T w: the flat one (true; *P rows a unit group, *VW elements a unit) or the columns. What bounds both is the
+// read of V. By single elements, for a V that is not 16-byte aligned, the flat form is the better one up to 32 columns, where
+// the column form leaves half of its 64 column threads idle (100k x 12 FP64: 62 us against 70, the whole product), and far worse
+// beyond (100k x 129 FP32: 47 us against 14). By 16-byte units, where its units occupy enough of the block's threads,
+//  - FP32 takes it (with the read of U after it, 100k x 177: 49 us against 55; 400k x 257: 172 against 226). Odd ranks from
+//    129 to 153, whose units of four rows leave 40 % of the threads idle, stay with the columns (100k x 129: 39
+//    against 35) unless V is too large for L2 (400k x 129: 118 against 137);
+//  - FP64, whose units hold two columns, gains up to 32 columns (400k x 12: 178 us against 211) and where V does not stay in
+//    L2 (400k x 257: 527 against 582); in between the columns are the faster ones (100k x 63: 76 against 80, 50k x 177: 88
+//    against 111).
+template <typename T>
+bool vtw_flat(const T* V, int64_t N, int rt, int* P, int* VW) {
+  *P = *VW = 1;
+  if ((reinterpret_cast<uintptr_t>(V) & 15) != 0) return rt <= 32;
+  constexpr int W = 16 / (int)sizeof(T);
+  *VW = W;
+  *P = rt % W == 0 ? 1 : W % 2 == 0 && (2 * rt) % W == 0 ? 2 : W;
+  const int nt = *P * rt / W, busy = nt >= 256 ? 256 : 256 / nt * nt;  // threads at work
+  const bool large = (double)N * rt * sizeof(T) > 129e6;
+  if (sizeof(T) == 4) return busy >= 154 || rt > 256 || large;
+  return rt <= 32 || (rt > 64 && busy >= 218 && large);
 }
 
 // t = sum over the partial rows, written into row 0 of `partial`: 32 columns x 8 part lanes
@@ -465,13 +536,13 @@ __global__ void __launch_bounds__(256) mt_kernel(const T* __restrict__ M, int rs
   if (lane == 0 && r < rs) s_out[r] = acc;
 }
 
-// out[p] = U[p, :] . s, a warp taking four consecutive rows at a time (their loads are all in
-// flight before any is reduced); s is read through the L1 cache. What bounds it: the read of U.
-// 100k x 177 FP32: 24.3 -> 18.8 us, 200k x 63: 23 -> 14.9 us, against one row at a time.
-template <typename T>
+// out[p] = U[p, :] . s, a warp taking R consecutive rows at a time (their loads are all in
+// flight before any is reduced); s is read through the L1 cache. What bounds it: the read of U. Four rows up to 128
+// columns, two beyond, on more blocks (four: 1M x 45 FP32 127 -> 140 us with two, the read of V before it included; two:
+// 50k x 516 FP32 143 -> 134, 5,000 x 180 FP64 31 -> 29).
+template <typename T, int R>
 __global__ void __launch_bounds__(256) us_kernel(const T* __restrict__ U, int64_t N, int rs,
                                                  const T* __restrict__ s, T* __restrict__ out) {
-  constexpr int R = 4;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t row = R * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); row < N; row += R * nw) {
@@ -497,7 +568,9 @@ __global__ void __launch_bounds__(256) us_kernel(const T* __restrict__ U, int64_
     }
 #pragma unroll
     for (int i = 0; i < R; ++i) acc[i] = warp_sum<T>(acc[i]);
-    if (lane < live) out[row + lane] = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+      if (lane == i && i < live) out[row + i] = acc[i];
   }
 }
 
@@ -508,13 +581,10 @@ pttk_status apply_typed(const T* U, const T* M, const T* V, int64_t N_s, int64_t
   T* sv = scratch + (size_t)nparts * rt;
   PTTK_PROF("apply", s);
   if (N_t > 0) {
-    constexpr int VW = 16 / (int)sizeof(T);
-    if ((reinterpret_cast<uintptr_t>(V) & 15) == 0) {
-      const int P = rt % VW == 0 ? 1 : VW % 2 == 0 && (2 * rt) % VW == 0 ? 2 : VW;
-      vtw_partial_kernel<T, VW><<<nparts, 256, 0, s>>>(V, N_t, rt, P, w, partial);
-    } else {
-      vtw_partial_kernel<T, 1><<<nparts, 256, 0, s>>>(V, N_t, rt, 1, w, partial);
-    }
+    int P, VW;
+    if (!vtw_flat(V, N_t, rt, &P, &VW)) vtw_columns_kernel<T><<<nparts, 256, 0, s>>>(V, N_t, rt, w, partial);
+    else if (VW == 1) vtw_flat_kernel<T, 1><<<nparts, 256, 0, s>>>(V, N_t, rt, P, w, partial);
+    else vtw_flat_kernel<T, 16 / (int)sizeof(T)><<<nparts, 256, 0, s>>>(V, N_t, rt, P, w, partial);
     pttk::count_launch();
   } else {
     PTTK_CUDA(cudaMemsetAsync(partial, 0, sizeof(T) * (size_t)nparts * rt, s));
@@ -526,8 +596,11 @@ pttk_status apply_typed(const T* U, const T* M, const T* V, int64_t N_s, int64_t
   }
   mt_kernel<T><<<(unsigned)((rs + 7) / 8), 256, 0, s>>>(M, rs, rt, partial, left, sv); pttk::count_launch();
   if (N_s > 0) {
-    const int64_t blocks = std::min<int64_t>((N_s * 8 + 255) / 256, (int64_t)sm_count() * 8);
-    us_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(U, N_s, rs, sv, out); pttk::count_launch();
+    const int R = rs <= 128 ? 4 : 2;
+    const unsigned blocks = (unsigned)std::min<int64_t>((N_s * (32 / R) + 255) / 256, (int64_t)sm_count() * (32 / R));
+    if (R == 4) us_kernel<T, 4><<<blocks, 256, 0, s>>>(U, N_s, rs, sv, out);
+    else us_kernel<T, 2><<<blocks, 256, 0, s>>>(U, N_s, rs, sv, out);
+    pttk::count_launch();
   }
   PTTK_CUDA(cudaGetLastError());
   return PTTK_OK;
