@@ -41,7 +41,7 @@
 namespace pttk {
 namespace {
 
-constexpr int RC = 1024;  // Householder rows per pass of the reflector through shared memory
+constexpr int RC = 4096;  // Householder rows per pass of the reflector through shared memory
 constexpr int HU = 8;     // rows per lane per load batch in the Householder passes
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -117,13 +117,18 @@ __global__ void transpose_kernel(const double* __restrict__ X, int64_t m, int64_
 // row comes exactly from the update of the previous step (per row group, summed in a fixed order), so
 // pivots and the stopping test use exact norms, not downdated ones.
 //
-// One cooperative launch per batch of matrices. A matrix has RG x CN blocks: block (rg, cb) owns the rows
-// of group rg and, 16 at a time, every CN-th set of columns (two per warp). A step is: dot products of the
+// One cooperative launch per batch of matrices. A matrix has RG x CN blocks: in each step block (rg, cb) takes the rows
+// of group rg and share cb of the columns left, 16 at a time (two per warp). A step is: dot products of the
 // reflector with the block's columns (partial per row group), a barrier among the matrix's blocks, the update with the
 // new norms, a barrier, and the pivot choice, which every block makes for itself from the same numbers. What
 // bounds it: 3 FP64 FMAs per remaining element and step where the matrix is large, two barriers a step
 // (about 5 us in all) where it is small. As five launches a step, the QRs of 20^5 took 15.8 ms,
 // now 4.0 (with the sectors).
+// The columns are dealt anew in each step: with a block keeping its columns for good, the warps whose columns were taken as
+// pivots stood idle (20736 x 3696, 1350 steps: 827 ms; five launches a step 575; now 571). Large batches run three blocks an SM
+// for the FP64 pipe (248832 x 756: 417 -> 402 ms), small ones two, since a barrier costs more with more blocks (3672 x 144: 3.5
+// against 5.1 ms); the line, 8 million elements, lies between 7281 x 729 (23.6 against 27.1 ms) and 10008 x 1728
+// (71.9 against 59.5).
 struct HHState {
   double tail2;  // ||R22||_F^2 at the stop (0 if every column was factored)
   int k;
@@ -192,8 +197,9 @@ struct QrBatch {
   int count;
 };
 
-__global__ void __launch_bounds__(256, 2) hh_kernel(QrBatch batch) {
-  extern __shared__ unsigned mask[];  // bit p: column p not yet factored
+template <int PER_SM>
+__global__ void __launch_bounds__(256, PER_SM) hh_kernel(QrBatch batch) {
+  extern __shared__ unsigned mask[];  // bit p: column p not yet factored; then the columns left before each word
   __shared__ double v[RC];
   __shared__ double s_tot[8], s_max[8], s_x0, s_below;
   __shared__ int s_arg[8];
@@ -207,7 +213,24 @@ __global__ void __launch_bounds__(256, 2) hh_kernel(QrBatch batch) {
   const int64_t M = jb.M, r_lo = M * rg / RG, r_hi = M * (rg + 1) / RG;
   double* __restrict__ A = jb.A;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int e = threadIdx.x; e < (N + 31) / 32; e += 256) mask[e] = 0xffffffffu;
+  const int nw = (N + 31) / 32;
+  int* before = reinterpret_cast<int*>(mask + nw);
+  for (int e = threadIdx.x; e < nw; e += 256) {
+    mask[e] = 32 * e + 32 <= N ? 0xffffffffu : (1u << (N & 31)) - 1u;
+    before[e] = 32 * e;
+  }
+  // physical column of the q-th one left, by a whole warp
+  auto column = [&](int q) -> int {
+    int w = -1;
+    for (int base = 0; base < nw; base += 32) {
+      const unsigned le = __ballot_sync(0xffffffffu, base + lane < nw && before[base + lane] <= q);
+      w += __popc(le);
+      if (le != 0xffffffffu) break;
+    }
+    const unsigned word = mask[w];
+    const bool hit = (word >> lane & 1u) && __popc(word & ((1u << lane) - 1u)) == q - before[w];
+    return 32 * w + __ffs(__ballot_sync(0xffffffffu, hit)) - 1;
+  };
   // squares below the first row, and the first row
   for (int c0 = cb * QC; c0 < N; c0 += CN * QC)
     for (int c = 0; c < 2; ++c) {
@@ -295,6 +318,7 @@ __global__ void __launch_bounds__(256, 2) hh_kernel(QrBatch batch) {
       tau = (beta - x0) / beta;
     }
     if (threadIdx.x == 0) mask[pj >> 5] &= ~(1u << (pj & 31));
+    for (int e = (pj >> 5) + 1 + threadIdx.x; e < nw; e += 256) --before[e];
     if (lb == 0 && threadIdx.x == 0) {
       jb.perm[j] = pj;
       jb.Rp[j + (int64_t)pj * N] = beta;
@@ -311,24 +335,25 @@ __global__ void __launch_bounds__(256, 2) hh_kernel(QrBatch batch) {
       for (int t = threadIdx.x; t < rows; t += 256) v[t] = lo + t == j ? 1.0 : __ldcg(vj + lo + t) * scale;
       __syncthreads();
     };
-    auto live = [&](int p) { return p < N && (mask[p >> 5] >> (p & 31) & 1u); };
-    for (int c0 = cb * QC; c0 < N; c0 += CN * QC) {
-      const int p0 = c0 + 2 * warp, p1 = p0 + 1;
-      const bool l0 = live(p0), l1 = live(p1);
-      const double* ca = A + (int64_t)(l0 ? p0 : p1) * M;
-      const double* cbp = A + (int64_t)(l1 ? p1 : p0) * M;
+    // this block's share of the columns left
+    const int left = N - 1 - j, q_lo = (int)((int64_t)left * cb / CN), q_hi = (int)((int64_t)left * (cb + 1) / CN);
+    for (int c0 = q_lo; c0 < q_hi; c0 += QC) {
+      const bool l0 = c0 + warp < q_hi, l1 = c0 + warp + 8 < q_hi;
+      const int p0 = l0 ? column(c0 + warp) : 0, p1 = l1 ? column(c0 + warp + 8) : 0;
+      const double* ca = A + (int64_t)p0 * M;
+      const double* cbp = A + (int64_t)p1 * M;
       double a0 = 0.0, a1 = 0.0;
       for (int64_t lo = b_lo; lo < r_hi; lo += RC) {
         const int rows = (int)std::min<int64_t>(RC, r_hi - lo);
         load_v(lo, rows);
-        if (!l0 && !l1) continue;
+        if (!l0) continue;
         for (int t0 = lane; t0 < rows; t0 += 32 * HU) {
           double x[HU], y[HU];  // all loads in flight before the arithmetic
 #pragma unroll
           for (int u = 0; u < HU; ++u) {
             const bool in = t0 + 32 * u < rows;
             x[u] = in ? __ldcg(ca + lo + t0 + 32 * u) : 0.0;
-            y[u] = in && l0 && l1 ? __ldcg(cbp + lo + t0 + 32 * u) : 0.0;
+            y[u] = in && l1 ? __ldcg(cbp + lo + t0 + 32 * u) : 0.0;
           }
 #pragma unroll
           for (int u = 0; u < HU; ++u) {
@@ -342,13 +367,13 @@ __global__ void __launch_bounds__(256, 2) hh_kernel(QrBatch batch) {
       a1 = warp_sum(a1);
       if (lane == 0) {
         if (l0) jb.wpart[(int64_t)rg * N + p0] = a0;
-        if (l1) jb.wpart[(int64_t)rg * N + p1] = l0 ? a1 : a0;
+        if (l1) jb.wpart[(int64_t)rg * N + p1] = a1;
       }
     }
     if (!grid_barrier(jb.sync, nblocks)) return;
-    for (int c0 = cb * QC; c0 < N; c0 += CN * QC) {
-      const int p0 = c0 + 2 * warp, p1 = p0 + 1;
-      const bool l0 = live(p0), l1 = live(p1);
+    for (int c0 = q_lo; c0 < q_hi; c0 += QC) {
+      const bool l0 = c0 + warp < q_hi, l1 = c0 + warp + 8 < q_hi;
+      const int p0 = l0 ? column(c0 + warp) : 0, p1 = l1 ? column(c0 + warp + 8) : 0;
       // w = tau sum over the row groups
       double w0 = 0.0, w1 = 0.0;
       for (int g = lane; g < RG; g += 32) {
@@ -358,34 +383,34 @@ __global__ void __launch_bounds__(256, 2) hh_kernel(QrBatch batch) {
       w0 = tau * warp_sum(w0);
       w1 = tau * warp_sum(w1);
       double n0 = 0.0, n1 = 0.0;
+      auto store = [&](double* col, int p, int64_t i, double a, double& nacc) {
+        *col = a;
+        if (i == j) jb.Rp[j + (int64_t)p * N] = a;
+        if (i == j + 1) jb.xrow[p] = a;
+        if (i >= j + 2) nacc = fma(a, a, nacc);
+      };
       for (int64_t lo = b_lo; lo < r_hi; lo += RC) {
         const int rows = (int)std::min<int64_t>(RC, r_hi - lo);
         if (!keep) load_v(lo, rows);
-        for (int c = 0; c < 2; ++c) {
-          if (!(c ? l1 : l0)) continue;
-          const int p = p0 + c;
-          const double wl = c ? w1 : w0;
-          double* col = A + (int64_t)p * M + lo;
-          double nacc = 0.0;
-          for (int t0 = lane; t0 < rows; t0 += 32 * HU) {
-            double x[HU];
+        if (!l0) continue;
+        double* ca = A + (int64_t)p0 * M + lo;
+        double* cbp = A + (int64_t)p1 * M + lo;
+        for (int t0 = lane; t0 < rows; t0 += 32 * HU) {
+          double x[HU], y[HU];
 #pragma unroll
-            for (int u = 0; u < HU; ++u) x[u] = t0 + 32 * u < rows ? __ldcg(col + t0 + 32 * u) : 0.0;
+          for (int u = 0; u < HU; ++u) {
+            const bool in = t0 + 32 * u < rows;
+            x[u] = in ? __ldcg(ca + t0 + 32 * u) : 0.0;
+            y[u] = in && l1 ? __ldcg(cbp + t0 + 32 * u) : 0.0;
+          }
 #pragma unroll
-            for (int u = 0; u < HU; ++u) {
-              const int t = t0 + 32 * u;
-              if (t < rows) {
-                const double a = fma(-v[t], wl, x[u]);
-                const int64_t i = lo + t;
-                col[t] = a;
-                if (i == j) jb.Rp[j + (int64_t)p * N] = a;
-                if (i == j + 1) jb.xrow[p] = a;
-                if (i >= j + 2) nacc = fma(a, a, nacc);
-              }
+          for (int u = 0; u < HU; ++u) {
+            const int t = t0 + 32 * u;
+            if (t < rows) {
+              store(ca + t, p0, lo + t, fma(-v[t], w0, x[u]), n0);
+              if (l1) store(cbp + t, p1, lo + t, fma(-v[t], w1, y[u]), n1);
             }
           }
-          if (c) n1 += nacc;
-          else n0 += nacc;
         }
       }
       n0 = warp_sum(n0);
@@ -836,15 +861,14 @@ pttk_status householder_batch(std::vector<Qr>& qr, cudaStream_t s) {
   const int count = (int)qr.size();
   int nmax = 1;
   for (const Qr& q : qr) nmax = std::max(nmax, q.N);
-  const size_t smem = sizeof(unsigned) * ((size_t)nmax + 31) / 32 + 16;
-  if (smem > 40 * 1024)
-    PTTK_CUDA(cudaFuncSetAttribute(hh_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int cap = 0;
-  PTTK_TRY(coop_capacity(hh_kernel, 256, smem, &cap));
-  // blocks in proportion to the elements, at least one per matrix: as many column sets as the share
-  // allows, then row groups of at least 64 rows
+  const size_t smem = (sizeof(unsigned) + sizeof(int)) * (((size_t)nmax + 31) / 32);
   double total = 0.0;
   for (const Qr& q : qr) total += (double)q.M * q.N;
+  auto kfn = total >= 8e6 ? hh_kernel<3> : hh_kernel<2>;
+  if (smem > 8 * 1024)
+    PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int cap = 0;
+  PTTK_TRY(coop_capacity(kfn, 256, smem, &cap));
   QrBatch b{};
   b.count = count;
   int next = 0;
@@ -858,8 +882,15 @@ pttk_status householder_batch(std::vector<Qr>& qr, cudaStream_t s) {
     j.Rp = qr[i].Rp;
     j.perm = qr[i].perm;
     const int share = std::max(1, (int)((double)(cap - count) * ((double)j.M * j.N / total)));
+    // a column set for each QC columns, and row groups of at least 64 rows; one group more, with fewer sets, where the sets
+    // leave over a fifth of the share idle (3696 columns: 231 sets in a share of 456)
     j.cn = std::max(1, std::min(share, (j.N + QC - 1) / QC));
-    j.rg = (int)std::max<int64_t>(1, std::min<int64_t>(share / j.cn, j.M / 64));
+    j.rg = share / j.cn;
+    if (5 * j.rg * j.cn < 4 * share) j.cn = share / ++j.rg;
+    if (j.rg > j.M / 64) {
+      j.rg = (int)std::max<int64_t>(1, j.M / 64);
+      j.cn = std::max(1, std::min(share / j.rg, (j.N + QC - 1) / QC));
+    }
     j.block0 = next;
     next += j.cn * j.rg;
     words += ((size_t)2 * j.rg + 1) * j.N;
@@ -882,7 +913,7 @@ pttk_status householder_batch(std::vector<Qr>& qr, cudaStream_t s) {
     PTTK_CUDA(cudaMemsetAsync(j.Rp, 0, sizeof(double) * (size_t)j.N * j.N, s));
   }
   void* args[] = {&b};
-  PTTK_CUDA(cudaLaunchCooperativeKernel((const void*)hh_kernel, dim3((unsigned)next), dim3(256), args, smem, s));
+  PTTK_CUDA(cudaLaunchCooperativeKernel((const void*)kfn, dim3((unsigned)next), dim3(256), args, smem, s));
   pttk::count_launch();
   std::vector<char> host(per * count);
   PTTK_CUDA(cudaMemcpyAsync(host.data(), sync.p, per * count, cudaMemcpyDeviceToHost, s));
