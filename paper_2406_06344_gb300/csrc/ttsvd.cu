@@ -1493,14 +1493,12 @@ pttk_status tt_svd_run(pttk_tt* tt, double* X, double tol, cudaStream_t s) {
     return dim >= 0 && (sym >> dim & 1u) ? (unsigned)(v & 1) << dim : 0u;
   };
 
-  Buf Xn;
-  PTTK_TRY(Xn.alloc(total, s));
   std::vector<Buf> cores(D);
   tt->ranks[0] = 1;
   int64_t r_prev = 1;
   std::vector<unsigned> qa(1, 0u);  // charges of the bond's values
-  double* cur = X;
-  double* nxt = Xn.p;
+  const double* cur = X;
+  Buf kept;  // the tensor after the first step, in cur
   int64_t cur_elems = total;
   for (int k = 0; k < D - 1; ++k) {
     const int64_t m = r_prev * n;
@@ -1583,14 +1581,17 @@ pttk_status tt_svd_run(pttk_tt* tt, double* X, double tol, cudaStream_t s) {
     }
     for (size_t i = 0; i < parts.size(); ++i) parts[i].r = (int)ids[i].size();
     PTTK_TRY(svd_finish(parts, clk, k, s));
-    // G_k, and X <- G_k^T X (r x c)
+    // G_k, and X <- G_k^T X (r x c), allocated only now that the QR inputs are gone: the sectors of an odd n are a little
+    // larger than the tensor's nonzero part, and both with the result took more than the two tensors of whole unfoldings
+    Buf nxt;
+    PTTK_TRY(nxt.alloc((int64_t)r * c, s));
     if (sym == 0) {
       cores[k] = std::move(parts[0].core);
-      dgemm(true, false, r, c, m, 1.0, cores[k].p, m, cur, m, 0.0, nxt, r, s);
+      dgemm(true, false, r, c, m, 1.0, cores[k].p, m, cur, m, 0.0, nxt.p, r, s);
     } else {
       PTTK_TRY(cores[k].alloc(m * r, s));
       PTTK_CUDA(cudaMemsetAsync(cores[k].p, 0, sizeof(double) * m * r, s));
-      PTTK_CUDA(cudaMemsetAsync(nxt, 0, sizeof(double) * r * c, s));
+      PTTK_CUDA(cudaMemsetAsync(nxt.p, 0, sizeof(double) * r * c, s));
       for (size_t i = 0; i < parts.size(); ++i) {
         SvdPart& pt = parts[i];
         if (pt.r == 0) continue;
@@ -1600,7 +1601,7 @@ pttk_status tt_svd_run(pttk_tt* tt, double* X, double tol, cudaStream_t s) {
         scatter_core_kernel<<<grid1d(pt.m * pt.r, 256), 256, 0, s>>>(pt.core.p, drows[i].ints(), (int)pt.m, dids.ints(), pt.r, m, cores[k].p); pttk::count_launch();
         PTTK_TRY(Y.alloc(pt.r * pt.c, s));
         dgemm(true, false, pt.r, pt.c, pt.m, 1.0, pt.core.p, pt.m, pt.X, pt.m, 0.0, Y.p, pt.r, s);
-        scatter_sector_kernel<<<grid1d(pt.c * 32, 256), 256, 0, s>>>(Y.p, pt.r, dids.ints(), r, cols[i], pt.c, nxt); pttk::count_launch();
+        scatter_sector_kernel<<<grid1d(pt.c * 32, 256), 256, 0, s>>>(Y.p, pt.r, dids.ints(), r, cols[i], pt.c, nxt.p); pttk::count_launch();
       }
       PTTK_CUDA(cudaStreamSynchronize(s));  // the host index lists have been read
     }
@@ -1608,7 +1609,8 @@ pttk_status tt_svd_run(pttk_tt* tt, double* X, double tol, cudaStream_t s) {
     clk.mark(k, "project");
     if (clk.on) fprintf(stderr, "pttk: tt-svd step %d rank %d\n", k + 1, r);
     tt->ranks[k + 1] = r;
-    std::swap(cur, nxt);
+    kept = std::move(nxt);
+    cur = kept.p;
     cur_elems = (int64_t)r * c;
     r_prev = r;
     qa = qn;
