@@ -65,7 +65,7 @@ cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s) {
       props.location.id = dev;
       cudaMemPool_t made = nullptr;
       cudaError_t e = cudaMemPoolCreate(&made, &props);
-      unsigned long long keep = kWorkspaceKeep;
+      unsigned long long keep = g_ws_handles > 0 ? kWorkspaceKeep : 0;
       if (e == cudaSuccess) e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
       if (e != cudaSuccess) {
         if (made) cudaMemPoolDestroy(made);
@@ -84,15 +84,22 @@ cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
-void ws_handle_added() {
-  std::lock_guard<std::mutex> lk(g_ws_mu);
-  ++g_ws_handles;
+// Under g_ws_mu, on the first and the last handle: what the pools keep from now on. A pool whose threshold falls to zero gives
+// back what finished work has left at once, and the rest at the next synchronisation after its release.
+static void ws_keep(unsigned long long bytes) {
+  for (cudaMemPool_t pool : g_ws_pool) {
+    if (!pool) continue;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes);
+    if (bytes == 0) cudaMemPoolTrimTo(pool, 0);
+  }
 }
-void ws_handle_freed() {
+WsHandle::WsHandle() {
   std::lock_guard<std::mutex> lk(g_ws_mu);
-  if (--g_ws_handles == 0)
-    for (cudaMemPool_t pool : g_ws_pool)
-      if (pool) cudaMemPoolTrimTo(pool, 0);
+  if (g_ws_handles++ == 0) ws_keep(kWorkspaceKeep);
+}
+WsHandle::~WsHandle() {
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  if (--g_ws_handles == 0) ws_keep(0);
 }
 
 // Target-side cores transposed to (right rank, j, left rank) so both factor chains read
@@ -113,8 +120,7 @@ __global__ void orient_kernel(const double* __restrict__ G, int ra, int n, int r
 
 // Handles keep their target-side oriented cores next to the cores (allocated together).
 struct pttk_tt_ext : pttk_tt {
-  pttk_tt_ext() { pttk::ws_handle_added(); }
-  ~pttk_tt_ext() { pttk::ws_handle_freed(); }
+  pttk::WsHandle ws;
   double* tgt64 = nullptr;
   float* tgt32 = nullptr;
   pttk::TcImageCache* tc = nullptr;  // tensor-core core images, built on first use per form

@@ -47,6 +47,7 @@ pttk_status transpose_rm(const double* in, int64_t rows, int64_t cols, double* o
 }  // namespace pttk
 
 struct pttk_fixed {
+  pttk::WsHandle ws;
   pttk_tt th;               // the rounded theta cores as a d = 0 handle (for Algorithm 3)
   int64_t Ns = 0, Nt = 0;
   double* S = nullptr;      // N_s x r_s', row-major

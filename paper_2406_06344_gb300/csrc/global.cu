@@ -25,6 +25,7 @@
 #include <numeric>
 
 struct pttk_global {
+  pttk::WsHandle ws;
   pttk_tt tt;          // metadata of the TT; tt.cores64 is a private copy of its FP64 cores
   int64_t N = 0;
   int rs = 0, rt = 0;  // r_d and r_{d+d_theta}: columns of S and of T

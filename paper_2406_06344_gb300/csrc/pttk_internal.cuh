@@ -67,17 +67,23 @@ int sm_count();
 // Stream-ordered scratch (freed with cudaFreeAsync) from the library's own memory pool of the current
 // device. The default pool gives all memory back at every synchronisation, so a caller that reads
 // each result paid for the mapping again in each call (220 us in an instantiate +
-// apply); this one keeps up to kWorkspaceKeep bytes until the last
-// handle is freed. While the stream is being captured, the default pool's graph allocations serve.
+// apply); this one keeps up to kWorkspaceKeep bytes while a handle lives (a tensor train, a Global or a Fixed), and nothing
+// beyond the next synchronisation when none does. What it keeps is not lost to the process: an allocation that
+// finds no other memory takes it (the driver's doing). While the stream is being captured, the default pool's graph
+// allocations serve.
 constexpr unsigned long long kWorkspaceKeep = 1ull << 30;
 cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s);
 template <typename T>
 inline cudaError_t ws_malloc(T** p, size_t bytes, cudaStream_t s) {
   return ws_malloc_bytes(reinterpret_cast<void**>(p), bytes, s);
 }
-// Counts the live handles (tensor trains); at zero the kept workspace is given back.
-void ws_handle_added();
-void ws_handle_freed();
+// A member of every handle: counts the live ones.
+struct WsHandle {
+  WsHandle();
+  ~WsHandle();
+  WsHandle(const WsHandle&) = delete;
+  WsHandle& operator=(const WsHandle&) = delete;
+};
 
 // Number of kernels the library has launched (every launch site increments it).
 void count_launch();
