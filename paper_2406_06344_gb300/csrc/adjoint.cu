@@ -548,7 +548,7 @@ template <typename T, int D, int RB>
 pttk_status launch_adj(const AdjArgs& a, const T* X, int64_t N, const T* w, T* dX, cudaStream_t s) {
   auto kfn = adj_reverse_kernel<T, D, RB>;
   const size_t smem = adj_smem<T>(D, a.n, a.r1, RB);
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   int per_sm = 1;
   PTTK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, AF_THREADS, smem));
   const int64_t blocks = std::min<int64_t>((N + AF_THREADS - 1) / AF_THREADS, (int64_t)sm_count() * std::max(per_sm, 1));

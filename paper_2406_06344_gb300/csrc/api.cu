@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -39,6 +40,26 @@ int sm_count() {
     count[dev] = c > 0 ? c : 1;
   }
   return count[dev];
+}
+
+cudaError_t allow_smem(const void* kernel) {
+  static std::mutex mu;
+  static std::map<const void*, int> room;  // what the kernel's static shared memory leaves of 227 KB: fixed by its code
+  int bytes = 0;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    const auto it = room.find(kernel);
+    if (it != room.end()) bytes = it->second;
+  }
+  if (bytes == 0) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    bytes = 227 * 1024 - (int)a.sharedSizeBytes;
+    std::lock_guard<std::mutex> lk(mu);
+    room[kernel] = bytes;
+  }
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 namespace {

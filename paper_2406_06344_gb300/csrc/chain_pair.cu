@@ -810,7 +810,7 @@ bool pair_plan(const pttk_tt* tt, pttk_prec prec, PairArgs& a, size_t* smem_out)
 template <int FMT, bool SPLIT>
 pttk_status launch_pair(const PairArgs& a, size_t smem, cudaStream_t s) {
   auto kfn = chain_pair_kernel<FMT, SPLIT>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   const int64_t clusters = std::max<int64_t>(1, std::min<int64_t>(a.npairs, sm_count() / 2));
   kfn<<<(unsigned)(2 * clusters), PAIR_THREADS, smem, s>>>(a);
   pttk::count_launch();

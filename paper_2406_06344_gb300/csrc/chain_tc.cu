@@ -2134,7 +2134,7 @@ static bool ts_plan(const pttk_tt* tt, const TcImageCache* cache, const Images& 
 template <int FMT, bool SPLIT, int NS>
 static pttk_status launch_ts(TsArgs a, int64_t T0, int64_t T1, size_t smem, cudaStream_t s) {
   auto kfn = chain_ts_kernel<FMT, SPLIT, NS>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   a.T0p = T0;
   a.nitems = T0 + T1;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(a.nitems, sm_count()));
@@ -2174,7 +2174,7 @@ static bool tse_plan(const pttk_tt* tt, const TcImageCache* cache, const Images&
 template <int FMT, bool SPLIT, int NSB>
 static pttk_status launch_tse(TsArgs a, int64_t T0, int64_t T1, size_t smem, cudaStream_t s) {
   auto kfn = chain_tse_kernel<FMT, SPLIT, NSB>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   a.T0p = T0;
   a.nitems = T0 + T1;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(a.nitems, sm_count()));
@@ -2215,7 +2215,7 @@ pttk_status tc_prepare(const pttk_tt* tt, TcImageCache* cache, pttk_prec prec, i
 template <int FMT, bool SPLIT, int KCB, int NS>
 static pttk_status launch_tc(const TcArgs& a, size_t smem, cudaStream_t s) {
   auto kfn = chain_tc_kernel<FMT, SPLIT, KCB, NS>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   const unsigned grid = (unsigned)std::min<int64_t>(a.ntiles, sm_count());
   kfn<<<grid, TC_THREADS, smem, s>>>(a); pttk::count_launch();
   PTTK_CUDA(cudaGetLastError());
@@ -2225,7 +2225,7 @@ static pttk_status launch_tc(const TcArgs& a, size_t smem, cudaStream_t s) {
 template <int FMT, bool SPLIT, int KCB, int NS>
 static pttk_status launch_tce(const TcArgs& a, size_t smem, cudaStream_t s) {
   auto kfn = chain_tce_kernel<FMT, SPLIT, KCB, NS>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   const unsigned grid = (unsigned)std::min<int64_t>(a.ntiles, sm_count());
   kfn<<<grid, TCE_THREADS, smem, s>>>(a); pttk::count_launch();
   PTTK_CUDA(cudaGetLastError());

@@ -397,7 +397,7 @@ pttk_status sym_eig_values(double* A, int k, int nb, double* d, double* e, doubl
     const size_t wv_bytes = sizeof(double) * 2 * (size_t)(k - 1);
     if (wv_bytes > 200 * 1024) return set_error(PTTK_ENOTSUP, "eigenproblem larger than 12800 x 12800");
     if (wv_bytes > 48 * 1024)
-      PTTK_CUDA(cudaFuncSetAttribute(w_rank2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wv_bytes));
+      PTTK_CUDA(allow_smem((const void*)w_rank2_kernel));
     const int nch_max = (k + CHUNK - 1) / CHUNK;
     double *part = nullptr, *vbuf = nullptr, *wbuf = nullptr;
     unsigned* done = nullptr;
@@ -480,7 +480,7 @@ pttk_status sym_eig_vectors(const double* A, const double* d, const double* e, c
   const size_t ii_bytes = sizeof(double) * 5 * (size_t)k + (size_t)k;
   const int in_smem = ii_bytes <= 200 * 1024;
   if (in_smem && ii_bytes > 48 * 1024)
-    PTTK_CUDA(cudaFuncSetAttribute(inverse_iteration_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ii_bytes));
+    PTTK_CUDA(allow_smem((const void*)inverse_iteration_kernel));
   PTTK_CUDA(ws_malloc(&work, in_smem ? sizeof(double) : sizeof(double) * 6 * (size_t)k * nclus, s));
   PTTK_CUDA(cudaMemcpyAsync(djob, job.data(), sizeof(int) * job.size(), cudaMemcpyHostToDevice, s));
   PTTK_CUDA(cudaMemcpyAsync(dz, sel_z.data(), sizeof(int) * nsel, cudaMemcpyHostToDevice, s));

@@ -302,7 +302,7 @@ pttk_status kv_sym_launch(int kind, const double* X, int64_t N, const KvArgs& k,
   const unsigned blocks = (unsigned)((int64_t)nS * (nS + 1) / 2);
   const size_t smem = sizeof(double) * S;
   auto kfn = T == 256 ? gp_kv_sym_kernel<D, 256> : gp_kv_sym_kernel<D, 64>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   kfn<<<blocks, T, smem, s>>>(kind, X, N, k, S, nS, v, part);
   return PTTK_OK;
 }

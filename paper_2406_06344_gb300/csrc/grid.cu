@@ -455,7 +455,7 @@ pttk_status launch_all(GridArgs a, T* C, cudaStream_t st) {
   const size_t smem = sizeof(T) * (a.tile + (size_t)a.D * a.n + 2 * (NB / 2) * (NB / 2) + 2 * a.n + FEXP_N +
                                     (a.kind == K_MATERN_NU ? KV_TABLE : 0));
   auto kfn = grid_tile_kernel<T, NB>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   int per_sm = 0;
   PTTK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, threads, smem));
   if (per_sm < 1) return set_error(PTTK_ENOTSUP, "grid tile does not fit on an SM");
@@ -479,7 +479,7 @@ pttk_status launch_all(GridArgs a, T* C, cudaStream_t st) {
     const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(64, 4096 / tin));
     const size_t smem_e = sizeof(T) * ((size_t)batch * tin + 2 * (NB / 2) * (NB / 2));
     auto efn = expand_kernel<T, NB>;
-    PTTK_CUDA(cudaFuncSetAttribute(efn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_e));
+    PTTK_CUDA(allow_smem((const void*)efn));
     const int64_t blocks = std::min<int64_t>((count + batch - 1) / batch, (int64_t)sm_count() * 16);
     PTTK_PROF("mode_transform", st);
     efn<<<(unsigned)blocks, 256, smem_e, st>>>(a, F, tin, tout, count, batch, C); pttk::count_launch();
@@ -542,7 +542,7 @@ pttk_status launch_entries(const GridArgs& a, const int* idx, int64_t M, T* out,
   const size_t smem = sizeof(T) * ((size_t)a.D * a.n + 2 * a.n +
                                    (a.kind == K_MATERN_NU ? KV_TABLE : 0));
   auto kfn = entries_kernel<T>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((M + 255) / 256, (int64_t)sm_count() * 8));
   PTTK_PROF("grid_entries", st);
   kfn<<<(unsigned)blocks, 256, smem, st>>>(a, idx, M, out, status); pttk::count_launch();

@@ -832,7 +832,7 @@ static pttk_status launch_chain(ChainArgs a, int ct_max, cudaStream_t s) {
   constexpr int P = 16 * TM;
   const size_t smem = sizeof(T) * ((size_t)2 * P * a.rin_max + (size_t)P * a.n + 2 * BK * P + 2 * BK * (ct_max + 2));
   auto kfn = ct_max <= 64 ? chain_kernel<T, TM, 64> : chain_kernel<T, TM, sizeof(T) == 8 ? 96 : 128>;
-  PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PTTK_CUDA(allow_smem((const void*)kfn));
   a.blocks0 = (a.side[0].N + P - 1) / P;
   const int64_t blocks = a.blocks0 + (a.side[1].N + P - 1) / P;
   PTTK_PROF("chain", s);

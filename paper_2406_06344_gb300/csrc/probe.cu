@@ -237,11 +237,11 @@ extern "C" pttk_status pttk_peak_probe(int kind, int64_t iters, void* stream, do
   PTTK_CUDA(cudaEventCreate(&e1));
   // the MMA loops take more than half an SM's shared memory (unused), so that no two of
   // their CTAs share an SM
-  PTTK_CUDA(cudaFuncSetAttribute(umma_loop_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaPadSmem));
-  PTTK_CUDA(cudaFuncSetAttribute(umma_loop_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaPadSmem));
-  PTTK_CUDA(cudaFuncSetAttribute(umma_stream_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem));
-  PTTK_CUDA(cudaFuncSetAttribute(umma_stream_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem));
-  PTTK_CUDA(cudaFuncSetAttribute(umma_stream_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem));
+  PTTK_CUDA(allow_smem((const void*)umma_loop_kernel<true>));
+  PTTK_CUDA(allow_smem((const void*)umma_loop_kernel<false>));
+  PTTK_CUDA(allow_smem((const void*)umma_stream_kernel<64>));
+  PTTK_CUDA(allow_smem((const void*)umma_stream_kernel<128>));
+  PTTK_CUDA(allow_smem((const void*)umma_stream_kernel<256>));
   double flops = 0.0;
   PTTK_CUDA(cudaEventRecord(e0, s));
   switch (kind) {

@@ -64,6 +64,11 @@ constexpr bool kDebugLog = false;
 
 int sm_count();
 
+// Lets a kernel take as much dynamic shared memory as a block can have, the same value on each call: with the size of the
+// launch at hand instead, another host thread's smaller launch of the same kernel could lower it in between,
+// and the launch was refused.
+cudaError_t allow_smem(const void* kernel);
+
 // Stream-ordered scratch (freed with cudaFreeAsync) from the library's own memory pool of the current
 // device. The default pool gives all memory back at every synchronisation, so a caller that reads
 // each result paid for the mapping again in each call (220 us in an instantiate +

@@ -866,7 +866,7 @@ pttk_status householder_batch(std::vector<Qr>& qr, cudaStream_t s) {
   for (const Qr& q : qr) total += (double)q.M * q.N;
   auto kfn = total >= 8e6 ? hh_kernel<3> : hh_kernel<2>;
   if (smem > 8 * 1024)
-    PTTK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    PTTK_CUDA(allow_smem((const void*)kfn));
   int cap = 0;
   PTTK_TRY(coop_capacity(kfn, 256, smem, &cap));
   QrBatch b{};
