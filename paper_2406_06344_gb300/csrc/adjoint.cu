@@ -346,11 +346,12 @@ __global__ void __launch_bounds__(256) chain_back_step(const T* __restrict__ X, 
 //   gbar_1[a] = sum_j T_j(x_2) Q[a, j],  dL/dx_1 = sum_{a,j} gbar_1[a] G_1[j, a] T_j'(x_1)
 // (d = 2 lacks the middle step, d = 1 has the last alone.) The rows G_2[a, j, :] sit in shared memory,
 // read as broadcasts; S_2 and gbar_2 (RB values, R_2 padded) in registers; the scalars that the loops
-// index (T_j(x_2), T_j'(x_2), S_1, gbar_1) in shared memory, one column per thread. About
+// index (T_j(x_2), the sums over a of S_1 Q, S_1, gbar_1) in shared memory, one column per thread. About
 // 11k FMAs a point at ranks 9, 44: at N = 500k, n = 12 the separate kernels (S_1, S_2, Q and gbar
-// in memory, shared-memory atomics per term) took 16.4 ms, this one 0.525 ms with scalar FP32 FMAs and 0.435 ms
+// in memory, shared-memory atomics per term) took 16.4 ms, this one 0.525 ms with scalar FP32 FMAs and 0.46 ms
 // with the two-wide ones. What bounds it: issue, and the FP64 pipe for the bases.
-// The bases are formed in FP64 and rounded to T.
+// The bases are formed in FP64 and rounded to T; the last sum of each derivative, over T_j', is in FP64 (T_j' and the terms
+// unrounded), as it is in the separate kernels.
 constexpr int AF_THREADS = 128;
 
 struct AdjArgs {
@@ -362,28 +363,33 @@ struct AdjArgs {
   const void* q;   // (R_in of the last step) x n, column-major
 };
 
-// T_j(x) and T_j'(x) dxhat/dx = j U_{j-1}(x) dxhat/dx, j < n, handed to f(j, t, dt)
-template <typename F>
+// T_j(x) (VALS) and T_j'(x) dxhat/dx = j U_{j-1}(x) dxhat/dx (DERIVS; else 0), j < n, handed to f(j, t, dt)
+template <bool VALS, bool DERIVS, typename F>
 __device__ __forceinline__ void cheb_each(double x, double lo, double hi, int n, F&& f) {
   const double xh = (2.0 * x - lo - hi) / (lo - hi), sc = 2.0 / (lo - hi), x2 = 2.0 * xh;
   double t0 = 1.0, t1 = xh, u0 = 0.0, u1 = sc, k = 1.0;
   f(0, 1.0, 0.0);
   for (int j = 1; j < n; ++j) {
-    f(j, t1, k * u1);
-    const double t2 = fma(x2, t1, -t0), u2 = fma(x2, u1, -u0);
-    t0 = t1;
-    t1 = t2;
-    u0 = u1;
-    u1 = u2;
-    k += 1.0;
+    f(j, VALS ? t1 : 0.0, DERIVS ? k * u1 : 0.0);
+    if (VALS) {
+      const double t2 = fma(x2, t1, -t0);
+      t0 = t1;
+      t1 = t2;
+    }
+    if (DERIVS) {
+      const double u2 = fma(x2, u1, -u0);
+      u0 = u1;
+      u1 = u2;
+      k += 1.0;
+    }
   }
 }
 
 template <typename T>
 size_t adj_smem(int d, int n, int r1, int rb) {
-  // G_1 (n x r1), q (n x rlast), G_2 (r1 n x rb), then per thread T_1', T_2, T_2' (n each), S_1, gbar_1 (r1 each)
+  // G_1 (n x r1), q (n x rlast), G_2 (r1 n x rb), then per thread T_2, E_2 (n each), S_1, gbar_1 (r1 each)
   const size_t shared = (size_t)n * r1 + (size_t)n * (d == 3 ? rb : d == 2 ? r1 : 1) + (d == 3 ? (size_t)r1 * n * rb : 0);
-  const size_t per = (size_t)3 * n + 2 * r1;
+  const size_t per = (size_t)2 * n + 2 * r1;
   return sizeof(T) * ((shared + 3) / 4 * 4 + per * AF_THREADS);
 }
 
@@ -444,9 +450,8 @@ __global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, cons
   const size_t shared = (size_t)n * r1 + (size_t)n * rl + (D == 3 ? (size_t)r1 * n * RB : 0);
   T* priv = reinterpret_cast<T*>(smem_raw) + (shared + 3) / 4 * 4 + tid;
   T* T2 = priv;                          // [j] at stride AF_THREADS
-  T* D2 = T2 + n * AF_THREADS;
-  T* D1 = D2 + n * AF_THREADS;
-  T* S1 = D1 + n * AF_THREADS;
+  T* E2 = T2 + n * AF_THREADS;           // [j]: sum over a of S_1[a] Q[a, j]
+  T* S1 = E2 + n * AF_THREADS;
   T* B1 = S1 + r1 * AF_THREADS;
   const int rlast = D == 3 ? a.r2 : D == 2 ? r1 : 1;
   if (D == 3)
@@ -470,21 +475,20 @@ __global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, cons
 #pragma unroll
     for (int i = 0; i < D; ++i) x[i] = (double)X[p * D + a.coord[i]];
     if constexpr (D == 1) {
-      T acc = T(0);
-      cheb_each(x[0], a.lo[0], a.hi[0], n, [&](int j, double, double dt) { acc = fma((T)dt, q[j], acc); });
-      dX[p] = acc * wp;
+      double acc = 0.0;
+      cheb_each<false, true>(x[0], a.lo[0], a.hi[0], n, [&](int j, double, double dt) { acc = fma(dt, widen(q[j]), acc); });
+      dX[p] = (T)(acc * widen(wp));
     } else {
       // S_1
       for (int al = 0; al < r1; ++al) S1[al * AF_THREADS] = T(0);
-      cheb_each(x[0], a.lo[0], a.hi[0], n, [&](int j, double t, double dt) {
+      cheb_each<true, false>(x[0], a.lo[0], a.hi[0], n, [&](int j, double t, double) {
         const T tj = (T)t;
-        D1[j * AF_THREADS] = (T)dt;
         for (int al = 0; al < r1; ++al) S1[al * AF_THREADS] = fma(tj, G1[al * n + j], S1[al * AF_THREADS]);
       });
       if constexpr (D == 3) {
-        cheb_each(x[1], a.lo[1], a.hi[1], n, [&](int j, double t, double dt) {
+        cheb_each<true, false>(x[1], a.lo[1], a.hi[1], n, [&](int j, double t, double) {
           T2[j * AF_THREADS] = (T)t;
-          D2[j * AF_THREADS] = (T)dt;
+          E2[j * AF_THREADS] = T(0);
         });
         T s2[RB], gb[RB];
 #pragma unroll
@@ -496,32 +500,32 @@ __global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, cons
             axpy<RB>(sa * T2[j * AF_THREADS], row, s2);
           }
         }
-        T dx3 = T(0);
-        cheb_each(x[2], a.lo[2], a.hi[2], n, [&](int j, double t, double dt) {
+        double dx3 = 0.0, dx2 = 0.0;
+        cheb_each<true, true>(x[2], a.lo[2], a.hi[2], n, [&](int j, double t, double dt) {
           const T tj = (T)t * wp;
           const T* row = q + j * RB;
           axpy<RB>(tj, row, gb);
-          dx3 = fma((T)dt, dot4<RB>(s2, row), dx3);
+          dx3 = fma(dt, widen(dot4<RB>(s2, row)), dx3);
         });
-        T dx2 = T(0);
         for (int al = 0; al < r1; ++al) {
           const T sa = S1[al * AF_THREADS];
           const T* row = G2 + (size_t)al * n * RB;
-          T g1a = T(0), da = T(0);
+          T g1a = T(0);
           for (int j = 0; j < n; ++j, row += RB) {
             const T qv = dot4<RB>(gb, row);
-            da = fma(D2[j * AF_THREADS], qv, da);
+            E2[j * AF_THREADS] = fma(sa, qv, E2[j * AF_THREADS]);
             g1a = fma(T2[j * AF_THREADS], qv, g1a);
           }
-          dx2 = fma(sa, da, dx2);
           B1[al * AF_THREADS] = g1a;
         }
-        dX[p * D + a.coord[2]] = dx3 * wp;
-        dX[p * D + a.coord[1]] = dx2;
+        cheb_each<false, true>(x[1], a.lo[1], a.hi[1], n,
+                               [&](int j, double, double dt) { dx2 = fma(dt, widen(E2[j * AF_THREADS]), dx2); });
+        dX[p * D + a.coord[2]] = (T)(dx3 * widen(wp));
+        dX[p * D + a.coord[1]] = (T)dx2;
       } else {
         for (int al = 0; al < r1; ++al) B1[al * AF_THREADS] = T(0);
-        T dx2 = T(0);
-        cheb_each(x[1], a.lo[1], a.hi[1], n, [&](int j, double t, double dt) {
+        double dx2 = 0.0;
+        cheb_each<true, true>(x[1], a.lo[1], a.hi[1], n, [&](int j, double t, double dt) {
           const T tj = (T)t * wp;
           const T* row = q + j * r1;
           T e = T(0);
@@ -529,17 +533,17 @@ __global__ void __launch_bounds__(AF_THREADS) adj_reverse_kernel(AdjArgs a, cons
             B1[al * AF_THREADS] = fma(tj, row[al], B1[al * AF_THREADS]);
             e = fma(S1[al * AF_THREADS], row[al], e);
           }
-          dx2 = fma((T)dt, e, dx2);
+          dx2 = fma(dt, widen(e), dx2);
         });
-        dX[p * D + a.coord[1]] = dx2 * wp;
+        dX[p * D + a.coord[1]] = (T)(dx2 * widen(wp));
       }
-      T dx1 = T(0);
-      for (int j = 0; j < n; ++j) {
+      double dx1 = 0.0;
+      cheb_each<false, true>(x[0], a.lo[0], a.hi[0], n, [&](int j, double, double dt) {
         T e = T(0);
         for (int al = 0; al < r1; ++al) e = fma(B1[al * AF_THREADS], G1[al * n + j], e);
-        dx1 = fma(D1[j * AF_THREADS], e, dx1);
-      }
-      dX[p * D + a.coord[0]] = dx1;
+        dx1 = fma(dt, widen(e), dx1);
+      });
+      dX[p * D + a.coord[0]] = (T)dx1;
     }
   }
 }
