@@ -86,7 +86,7 @@ cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s) {
       props.location.id = dev;
       cudaMemPool_t made = nullptr;
       cudaError_t e = cudaMemPoolCreate(&made, &props);
-      unsigned long long keep = g_ws_handles > 0 ? kWorkspaceKeep : 0;
+      unsigned long long keep = g_ws_handles > 0 ? kWorkspaceKeep : kWorkspaceIdle;
       if (e == cudaSuccess) e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
       if (e != cudaSuccess) {
         if (made) cudaMemPoolDestroy(made);
@@ -105,13 +105,13 @@ cudaError_t ws_malloc_bytes(void** p, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
-// Under g_ws_mu, on the first and the last handle: what the pools keep from now on. A pool whose threshold falls to zero gives
-// back what finished work has left at once, and the rest at the next synchronisation after its release.
+// Under g_ws_mu, on the first and the last handle: what the pools keep from now on. A pool whose threshold falls gives back what
+// finished work has left at once, and the rest at the next synchronisation after its release.
 static void ws_keep(unsigned long long bytes) {
   for (cudaMemPool_t pool : g_ws_pool) {
     if (!pool) continue;
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes);
-    if (bytes == 0) cudaMemPoolTrimTo(pool, 0);
+    cudaMemPoolTrimTo(pool, bytes);
   }
 }
 WsHandle::WsHandle() {
@@ -120,7 +120,7 @@ WsHandle::WsHandle() {
 }
 WsHandle::~WsHandle() {
   std::lock_guard<std::mutex> lk(g_ws_mu);
-  if (--g_ws_handles == 0) ws_keep(0);
+  if (--g_ws_handles == 0) ws_keep(kWorkspaceIdle);
 }
 
 // Target-side cores transposed to (right rank, j, left rank) so both factor chains read

@@ -1,5 +1,6 @@
-"""The library keeps workspace between calls (up to 1 GiB) only while a handle lives. Each case runs in a process of its own,
-and compares the free memory (within a granule of 32 MiB) before a call and after it and a synchronisation."""
+"""The library keeps workspace between calls (up to 1 GiB) only while a handle lives, and 32 MiB otherwise. Each case runs in a
+process of its own, and compares the free memory (within one granule of 32 MiB) before a call and after it and a
+synchronisation."""
 import os
 import subprocess
 import sys
