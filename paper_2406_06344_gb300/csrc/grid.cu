@@ -23,6 +23,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "fexp.cuh"
 #include "kernels.cuh"
@@ -34,6 +35,8 @@ namespace {
 struct GridArgs {
   int kind, d, dtheta, D, n, m1;
   int64_t tile, ntiles;
+  int parts;             // threads that share the length scales of one point pair (grid_tile_kernel)
+  int direct;            // kappa_l for every entry: FP32, kernels without a fast form, and scales whose inverse overflows
   int ext[PTTK_MAX_D];   // carried extent of each mode: n, or (n + 1) / 2 for a folded source mode
   double lo[PTTK_MAX_D], hi[PTTK_MAX_D];
   // general-nu Matern, grid tile kernel: per nu node, G(z) = z^nu e^z K_nu(z) on [kv_zlo, kv_zhi]
@@ -64,7 +67,10 @@ constexpr int KV_MAX_PIECES = 64;
 // One block per nu node: the pieces' values at their Chebyshev points, the coefficients
 // c_m = (2 / (KV_DEG + 1)) sum_k G(z_k) T_m(zeta_k) (c_0 halved), then the powers' coefficients; FP64 and an
 // FP32 copy.
-__global__ void __launch_bounds__(256) kv_table_kernel(int n, int P, double zlo, double nu_lo, double nu_hi,
+struct KvBasis {
+  double t[KV_DEG + 1][KV_DEG + 1];  // t[k][q]: coefficient of t^q in T_k
+};
+__global__ void __launch_bounds__(256) kv_table_kernel(int n, int P, double zlo, double nu_lo, double nu_hi, KvBasis basis,
                                                        double* __restrict__ tab64, float* __restrict__ tab32) {
   __shared__ double stab[KV_TABLE];
   __shared__ double vals[KV_MAX_PIECES * (KV_DEG + 1)];
@@ -98,24 +104,10 @@ __global__ void __launch_bounds__(256) kv_table_kernel(int n, int P, double zlo,
     } else if (m == 1) {
       v = 2.0 / (b - a);
     } else {
-      // coefficient of t^q in sum_k c_k T_k(t): T_k = (k / 2) sum_j (-1)^j (k - j - 1)! / (j! (k - 2 j)!) (2 t)^(k - 2 j)
+      // coefficient of t^q in sum_k c_k T_k(t)
       const int q = m - 2;
       v = 0.0;
-      for (int k = KV_DEG - ((KV_DEG - q) & 1); k >= q; k -= 2) {
-        double w = 1.0;
-        if (k > 0) {
-          const int j = (k - q) / 2;
-          // (k / 2) (k - j - 1)! / (j! q!) 2^q, as a product of ratios (all intermediate values are exact or nearly so)
-          w = 0.5 * k;
-          for (int i = 1; i <= q; ++i) w *= 2.0;
-          // (k - j - 1)! / q! = (q + 1) ... (k - j - 1) = j - 1 factors for j >= 1, 1 / q for j = 0
-          if (j == 0) w /= q;
-          for (int i = q + 1; i <= k - j - 1; ++i) w *= i;
-          for (int i = 2; i <= j; ++i) w /= i;
-          if (j & 1) w = -w;
-        }
-        v = fma(w, cheb[p * (KV_DEG + 1) + k], v);
-      }
+      for (int k = KV_DEG - ((KV_DEG - q) & 1); k >= q; k -= 2) v = fma(basis.t[k][q], cheb[p * (KV_DEG + 1) + k], v);
     }
     tab64[((size_t)inu * P + p) * KV_STRIDE + m] = v;
     tab32[((size_t)inu * P + p) * KV_STRIDE + m] = (float)v;
@@ -149,7 +141,7 @@ __device__ __forceinline__ T kappa_matern_nu_tab(const GridArgs& a, int inu, T r
   return kappa_matern_nu_slow<T>(r2, l, nu, cnu, snu, stab);
 }
 
-// The closed forms from r^2 and r = sqrt(r^2), in FP64 with the table exponential.
+// Four closed forms from r^2 and r = sqrt(r^2), in FP64 with the table exponential (GridArgs::direct is 0 for these alone).
 __device__ __forceinline__ double kappa_r(int kind, double r2, double r, double l, double invl, const double* __restrict__ ftab) {
   switch (kind) {
     case K_GAUSS: return fexp_neg(r2 * invl * invl, ftab);
@@ -165,6 +157,7 @@ __device__ __forceinline__ double kappa_r(int kind, double r2, double r, double 
     default: return kappa_l<double>(kind, r2, l);
   }
 }
+// never taken in FP32
 __device__ __forceinline__ float kappa_r(int kind, float r2, float, float l, float, const float*) {
   return kappa_l<float>(kind, r2, l);
 }
@@ -234,7 +227,9 @@ __device__ __forceinline__ void transform_fibre(const T* __restrict__ Ah, int n,
     ev[i] = lo + hi;
     od[i] = 2 * i + 1 < n ? lo - hi : T(0);
   }
-#pragma unroll
+  // One pair of rows at a time: unrolled, the compiler keeps rows of Ah in registers across fibres and spills (20^6 general-nu
+  // Matern 13.7 -> 12.9 ms in FP64, with the other changes 2.65 -> 1.22 ms in FP32).
+#pragma unroll 1
   for (int m = 0; m < NBH; ++m) {
     T ye = T(0), yo = T(0);
 #pragma unroll
@@ -259,7 +254,8 @@ __global__ void __launch_bounds__(512) grid_tile_kernel(GridArgs a, T* __restric
   T* stab = ftab + FEXP_N;
   fill_tables<T>(a, eta, cnu, snu, stab);
   fill_half<T, NB>(a.n, Ah);
-  if constexpr (sizeof(T) == 8) fexp_fill(ftab);
+  if constexpr (sizeof(T) == 8)
+    if (!a.direct) fexp_fill(ftab);
   __syncthreads();
 
   const int n = a.n, d = a.d, dth = a.dtheta, m1 = a.m1;
@@ -267,9 +263,10 @@ __global__ void __launch_bounds__(512) grid_tile_kernel(GridArgs a, T* __restric
   // them all when that mode lies in the tile
   const bool inner = dth > 0 && m1 > d;
   const int nq = inner ? n : 1;
-  int64_t sx = 1;  // stride of the first parameter's mode in the tile
-  for (int j = 0; j < std::min(m1, d); ++j) sx *= a.ext[j];
-  const int64_t groups = a.tile / nq;
+  int sx = 1;  // stride of the first parameter's mode in the tile
+  for (int j = 0; j < min(m1, d); ++j) sx *= a.ext[j];
+  const int tile_n = (int)a.tile, groups = tile_n / nq;
+  const int per = (nq + a.parts - 1) / a.parts;
   for (int64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
     int idx[PTTK_MAX_D];
     int64_t rem = t;
@@ -277,37 +274,44 @@ __global__ void __launch_bounds__(512) grid_tile_kernel(GridArgs a, T* __restric
       idx[j] = (int)(rem % a.ext[j]);
       rem /= a.ext[j];
     }
-    for (int64_t g = threadIdx.x; g < groups; g += blockDim.x) {
-      int64_t q = g;
+    for (int it = threadIdx.x; it < groups * a.parts; it += blockDim.x) {
+      const int part = it / groups, g = it - part * groups;
+      const int li0 = part * per, li1 = min(nq, li0 + per);
+      int q = g;
       for (int j = 0; j < m1; ++j) {
         if (inner && j == d) continue;
-        idx[j] = (int)(q % a.ext[j]);
-        q /= a.ext[j];
+        const int next = q / a.ext[j];
+        idx[j] = q - next * a.ext[j];
+        q = next;
       }
       T r2 = T(0);
       for (int j = 0; j < d; ++j) {
         const T diff = eta[j * n + idx[j]] - eta[(d + dth + j) * n + idx[d + dth + j]];
         r2 += diff * diff;
       }
-      const T r = sqrt(r2);
-      T* dst = tile + (inner ? g % sx + (g / sx) * sx * n : g);
+      T* dst = tile + (inner ? g % sx + (g / sx) * sx * n + li0 * sx : g);
       const int l0 = inner ? 0 : dth > 0 ? idx[d] : 0;
       const int inu = dth > 1 ? idx[d + 1] : 0;
-      for (int li = 0; li < nq; ++li, dst += sx) {
-        const T l = dth > 0 ? eta[d * n + l0 + li] : T(1);
-        const T invl = T(1) / l;
-        *dst = a.kind == K_MATERN_NU
-                   ? kappa_matern_nu_tab<T>(a, inu, r2, r, l, invl, eta[(d + 1) * n + inu], cnu[inu], snu[inu], stab, ftab)
-                   : kappa_r(a.kind, r2, r, l, invl, ftab);
+      if (a.direct) {
+        for (int li = li0; li < li1; ++li, dst += sx) *dst = kappa_l<T>(a.kind, r2, dth > 0 ? eta[d * n + l0 + li] : T(1));
+      } else {
+        const T r = sqrt(r2);
+        for (int li = li0; li < li1; ++li, dst += sx) {
+          const T l = eta[d * n + l0 + li];
+          const T invl = T(1) / l;
+          *dst = a.kind == K_MATERN_NU
+                     ? kappa_matern_nu_tab<T>(a, inu, r2, r, l, invl, eta[(d + 1) * n + inu], cnu[inu], snu[inu], stab, ftab)
+                     : kappa_r(a.kind, r2, r, l, invl, ftab);
+        }
       }
     }
     __syncthreads();
     // the tile's unfolded modes: one fibre per thread
-    int64_t s = 1;
-    for (int j = 0; j < m1; s *= a.ext[j], ++j) {
+    int st = 1;
+    for (int j = 0; j < m1; st *= a.ext[j], ++j) {
       if (a.ext[j] != n) continue;
-      const int64_t nfib = a.tile / n;
-      for (int64_t f = threadIdx.x; f < nfib; f += blockDim.x) transform_fibre<T, NB>(Ah, n, tile + f % s + f / s * s * n, s);
+      const int nfib = tile_n / n;
+      for (int f = threadIdx.x; f < nfib; f += blockDim.x) transform_fibre<T, NB>(Ah, n, tile + f % st + f / st * st * n, (int64_t)st);
       __syncthreads();
     }
     T* out = C + t * a.tile;
@@ -370,7 +374,7 @@ __global__ void __launch_bounds__(256) expand_kernel(GridArgs a, const T* __rest
           const T v = i < nh ? base[i * s] : T(0);
           x[i] = 2 * i + 1 == n ? v : v + v;
         }
-#pragma unroll
+#pragma unroll 1
         for (int h = 0; h < NBH; ++h) {
           T y = T(0);
 #pragma unroll
@@ -410,12 +414,16 @@ void plan_tiles(GridArgs& a, bool fold, size_t elem) {
     if (a.lo[j] + a.hi[j] == a.lo[a.d + a.dtheta + j] + a.hi[a.d + a.dtheta + j]) a.ext[j] = (a.n + 1) / 2;
   a.m1 = 1;
   a.tile = a.ext[0];
-  while (a.m1 < a.D && (size_t)(a.tile * a.ext[a.m1]) * elem <= budget) {
+  a.ntiles = 1;
+  for (int j = 1; j < a.D; ++j) a.ntiles *= a.ext[j];
+  // A tile above 4096 entries only where that leaves every fourth SM one: a small grid in one tile is one block's work (32^3, boxes
+  // equal, thin-plate spline FP64: 424 us in one tile, 155 in 32).
+  while (a.m1 < a.D && (size_t)(a.tile * a.ext[a.m1]) * elem <= budget &&
+         (a.tile * a.ext[a.m1] <= 4096 || a.ntiles / a.ext[a.m1] >= sm_count() / 4)) {
+    a.ntiles /= a.ext[a.m1];
     a.tile *= a.ext[a.m1];
     ++a.m1;
   }
-  a.ntiles = 1;
-  for (int j = a.m1; j < a.D; ++j) a.ntiles *= a.ext[j];
 }
 
 template <typename T, int NB>
@@ -452,6 +460,18 @@ pttk_status launch_all(GridArgs a, T* C, cudaStream_t st) {
     }
   }
   const int threads = sizeof(T) == 8 ? 512 : 256;
+  // The length scales of a point pair over `parts` threads: the fewest rounds of the block, each counted as its evaluations
+  // and 0.4 for r (20^6 FP32: 400 pairs for 256 threads, 20 scales each, 78 % of the block busy; in 5 parts 98 %).
+  a.parts = 1;
+  if (a.dtheta > 0 && a.m1 > a.d) {
+    double least = 0.0;
+    for (int p = 1; p <= a.n; ++p) {
+      const double cost = (double)((a.tile / a.n * p + threads - 1) / threads) * ((a.n + p - 1) / p + 0.4);
+      if (p > 1 && cost >= least) continue;
+      least = cost;
+      a.parts = p;
+    }
+  }
   const size_t smem = sizeof(T) * (a.tile + (size_t)a.D * a.n + 2 * (NB / 2) * (NB / 2) + 2 * a.n + FEXP_N +
                                     (a.kind == K_MATERN_NU ? KV_TABLE : 0));
   auto kfn = grid_tile_kernel<T, NB>;
@@ -476,7 +496,9 @@ pttk_status launch_all(GridArgs a, T* C, cudaStream_t st) {
   }
   if (folded != total) {
     const int64_t count = total / tout;
-    const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(64, 4096 / tin));
+    // about 4096 values a block at a time, fewer where that leaves SMs without a block (9^6 FP64: 381 us with 18 indices a
+    // block, 81 with 1)
+    const int batch = (int)std::max<int64_t>(1, std::min<int64_t>({64, 4096 / tin, count / ((int64_t)sm_count() * 4)}));
     const size_t smem_e = sizeof(T) * ((size_t)batch * tin + 2 * (NB / 2) * (NB / 2));
     auto efn = expand_kernel<T, NB>;
     PTTK_CUDA(allow_smem((const void*)efn));
@@ -582,6 +604,8 @@ pttk_status grid_coeffs_launch(int kernel, int d, int dtheta, int n, const doubl
     a.lo[j] = box[j][0];
     a.hi[j] = box[j][1];
   }
+  const bool closed = kernel == K_GAUSS || kernel == K_MATERN32 || kernel == K_EXPONENTIAL || kernel == K_MATERN52;
+  a.direct = kernel != K_MATERN_NU && !(closed && fp64 && std::isfinite(1.0 / a.lo[d]));
   plan_tiles(a, true, fp64 ? 8 : 4);
   // the per-nu tables live until the kernels that read them have run: released stream-ordered
   // on every return path
@@ -633,7 +657,11 @@ pttk_status grid_coeffs_launch(int kernel, int d, int dtheta, int n, const doubl
       const size_t cnt = (size_t)n * P * KV_STRIDE;
       PTTK_CUDA(ws_malloc(&tab64, sizeof(double) * cnt, s));
       PTTK_CUDA(ws_malloc(&tab32, sizeof(float) * cnt, s));
-      kv_table_kernel<<<n, 256, 0, s>>>(n, P, zlo, a.lo[d + 1], a.hi[d + 1], tab64, tab32); pttk::count_launch();
+      KvBasis basis{};  // T_{k+1} = 2 t T_k - T_{k-1}, exact integers
+      basis.t[0][0] = basis.t[1][1] = 1.0;
+      for (int k = 2; k <= KV_DEG; ++k)
+        for (int q = 0; q <= k; ++q) basis.t[k][q] = (q > 0 ? 2.0 * basis.t[k - 1][q - 1] : 0.0) - basis.t[k - 2][q];
+      kv_table_kernel<<<n, 256, 0, s>>>(n, P, zlo, a.lo[d + 1], a.hi[d + 1], basis, tab64, tab32); pttk::count_launch();
       PTTK_CUDA(cudaGetLastError());
       a.kv_tab = fp64 ? static_cast<const void*>(tab64) : static_cast<const void*>(tab32);
       a.kv_P = P;
