@@ -279,11 +279,18 @@ int kv_splits(int64_t N) {
   return (int)std::min<int64_t>({want, 64, (N + GTILE - 1) / GTILE});
 }
 
-// The symmetric form serves FP64 products up to about 2.3 million points (its column sums in shared memory).
-bool kv_symmetric(int64_t N, bool fp32) {
+KvArgs kv_args(int kind, double l) {
+  const double c = kind == PTTK_MATERN32 ? 1.7320508075688772 : kind == PTTK_MATERN52 ? 2.23606797749979 : 1.0;
+  return KvArgs{l, -64.0 / (0.69314718055994530942 * l * l), c / l, 1010.0 * 0.69314718055994530942 * l * l};
+}
+
+// The symmetric form serves FP64 products up to about 2.3 million points (its column sums in shared memory), with length
+// scales whose factors are finite (times r = 0 an infinite one gives NaN where the division gives 0).
+bool kv_symmetric(int kind, double l, int64_t N, bool fp32) {
   int T, S, nS;
   kv_sym_shape(N, &T, &S, &nS);
-  return !fp32 && S <= 24576;
+  const KvArgs k = kv_args(kind, l);
+  return !fp32 && S <= 24576 && std::isfinite(kind == PTTK_GAUSS ? k.s : k.cl);
 }
 
 // doubles of scratch for one product (sym: the symmetric form)
@@ -321,8 +328,7 @@ pttk_status kv_launch(int kind, int d, const double* X, int64_t N, double l, dou
   } else {
     int T, S;
     kv_sym_shape(N, &T, &S, &ncs);
-    const double c = kind == PTTK_MATERN32 ? 1.7320508075688772 : kind == PTTK_MATERN52 ? 2.23606797749979 : 1.0;
-    const KvArgs k{l, -64.0 / (0.69314718055994530942 * l * l), c / l, 1010.0 * 0.69314718055994530942 * l * l};
+    const KvArgs k = kv_args(kind, l);
     switch (d) {
       case 1: PTTK_TRY(kv_sym_launch<1>(kind, X, N, k, v, part, s)); break;
       case 2: PTTK_TRY(kv_sym_launch<2>(kind, X, N, k, v, part, s)); break;
@@ -380,7 +386,7 @@ pttk_status pttk_gp_kv(int kernel, int d, const double* X, int64_t N, const doub
   if (prec != PTTK_FP64 && prec != PTTK_FP32) return set_error(PTTK_EINVAL, "K v: prec must be PTTK_FP64 or PTTK_FP32");
   cudaStream_t s = as_stream(stream);
   double* part = nullptr;
-  bool sym = kv_symmetric(N, prec == PTTK_FP32);
+  bool sym = kv_symmetric(kernel, theta[0], N, prec == PTTK_FP32);
   if (sym && ws_malloc(&part, sizeof(double) * kv_part_elems(N, true), s) != cudaSuccess) {
     cudaGetLastError();  // the general form needs less scratch
     sym = false;
@@ -412,7 +418,7 @@ pttk_status pttk_gp_pcg(int kernel, int d, const double* X, int64_t N, const dou
   PTTK_TRY(sc.get(&Ap, N));
   PTTK_TRY(sc.get(&part, nparts));
   double* kvpart = nullptr;
-  bool sym = kv_symmetric(N, prec == PTTK_FP32);
+  bool sym = kv_symmetric(kernel, theta[0], N, prec == PTTK_FP32);
   if (sym && sc.get(&kvpart, kv_part_elems(N, true)) != PTTK_OK) {
     cudaGetLastError();
     clear_error();
