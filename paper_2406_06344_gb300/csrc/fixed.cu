@@ -112,13 +112,19 @@ pttk_status pttk_fixed_create(const pttk_tt* tt, const double* X, int64_t N_s, c
   for (int j = 0; j <= dth; ++j) ranks[j] = tt->ranks[d + j];
   std::vector<double*> G(dth + 2, nullptr);
   std::vector<int> nr(dth + 1);
-  if (tol > 0.0) {
+  // Phase 4's arrays are scratch of the pool, which cudaFree would release without waiting for work that reads it: they go in
+  // stream order, and the handle keeps a copy of T'
+  const bool pooled = tol > 0.0;
+  auto drop = [&](double* q) {
+    if (q && pooled) cudaFreeAsync(q, s);
+    else if (q) cudaFree(q);
+  };
+  if (pooled) {
     // Phase 4
     const pttk_status st = phase4_round(Scol, N_s, thc.data(), ranks.data(), n, dth, V, N_t, tol, G.data(),
                                         nr.data(), s);
     if (st != PTTK_OK) {
-      for (double* q : G)
-        if (q) cudaFree(q);
+      for (double* q : G) drop(q);
       return st;
     }
   } else {
@@ -165,12 +171,17 @@ pttk_status pttk_fixed_create(const pttk_tt* tt, const double* X, int64_t N_s, c
   if (e == cudaSuccess) e = cudaMalloc(&f->S, sizeof(double) * (size_t)N_s * nr[0]);
   if (e == cudaSuccess) res = transpose_rm(G[0], nr[0], N_s, f->S, s);  // (r_s' x N_s row-major)^T
   if (e == cudaSuccess && res == PTTK_OK) {
-    f->T = G[dth + 1];
-    G[dth + 1] = nullptr;
-    e = cudaStreamSynchronize(s);
+    if (pooled) {
+      const size_t bytes = sizeof(double) * (size_t)N_t * nr[dth];
+      e = cudaMalloc(&f->T, bytes);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(f->T, G[dth + 1], bytes, cudaMemcpyDeviceToDevice, s);
+    } else {
+      f->T = G[dth + 1];
+      G[dth + 1] = nullptr;
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  for (int j = 0; j < dth + 1; ++j)
-    if (G[j]) cudaFree(G[j]);
+  for (double* q : G) drop(q);
   if (e != cudaSuccess || res != PTTK_OK) {
     fixed_release(f);
     return e != cudaSuccess ? cuda_error(e, "Phase 4 handle") : res;

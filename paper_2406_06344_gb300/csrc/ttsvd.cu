@@ -1695,21 +1695,13 @@ pttk_status tt_round_run(const pttk_tt* in, double tol, pttk_tt* out, cudaStream
   return pack_cores(out, G, s);
 }
 
-// *out: a cudaMalloc'd copy of b. Results that a handle or a caller keeps are such arrays and no scratch from the pool:
-// cudaFree waits for work that still reads the former, and does not for the latter.
-static pttk_status owned_copy(const Buf& b, int64_t elems, double** out, cudaStream_t s) {
-  PTTK_CUDA(cudaMalloc(out, sizeof(double) * std::max<int64_t>(elems, 1)));
-  PTTK_CUDA(cudaMemcpyAsync(*out, b.p, sizeof(double) * elems, cudaMemcpyDeviceToDevice, s));
-  return PTTK_OK;
-}
-
 // Phase 4 of Algorithm 2: TT-Round of [T^(1)(S), G_{d+1}, .., G_{d+d_theta}, T^(3)(T^T)]
 // (Eq. twist). Scol: N_s x r_s column-major (the first core 1 x N_s x r_s); theta cores
 // ranks[j] x n x ranks[j+1], j < d_theta (ranks[0] = r_s, ranks[d_theta] = r_t); Tt: r_t x N_t
 // column-major (the last core r_t x N_t x 1, i.e. T row-major). Inputs are not modified. On
 // return out[0] (N_s x r_s' column-major), out[1 .. d_theta] (the rounded theta cores) and
-// out[d_theta + 1] (r_t' x N_t column-major) are cudaMalloc'd arrays the caller frees, and
-// new_ranks[0 .. d_theta] their ranks. Synchronises `s`.
+// out[d_theta + 1] (r_t' x N_t column-major) are blocks of the workspace pool that the caller frees with cudaFreeAsync on `s`
+// (and copies what it keeps), and new_ranks[0 .. d_theta] their ranks. Synchronises `s`.
 pttk_status phase4_round(const double* Scol, int64_t Ns, const double* const* theta_cores, const int* ranks, int n,
                          int dtheta, const double* Tt, int64_t Nt, double tol, double** out, int* new_ranks,
                          cudaStream_t s) {
@@ -1728,8 +1720,10 @@ pttk_status phase4_round(const double* Scol, int64_t Ns, const double* const* th
     PTTK_CUDA(cudaMemcpyAsync(G[k].p, src, sizeof(double) * e, cudaMemcpyDeviceToDevice, s));
   }
   PTTK_TRY(tt_round_cores(G, r, nm, tol, s));
-  for (int k = 0; k < D; ++k) PTTK_TRY(owned_copy(G[k], r[k] * nm[k] * r[k + 1], &out[k], s));
-  PTTK_CUDA(cudaStreamSynchronize(s));
+  for (int k = 0; k < D; ++k) {
+    out[k] = G[k].p;
+    G[k].p = nullptr;
+  }
   for (int j = 0; j <= dtheta; ++j) new_ranks[j] = (int)r[j + 1];
   return PTTK_OK;
 }
@@ -1741,7 +1735,10 @@ pttk_status range_basis(const double* X, int64_t m, int64_t c, double** basis, i
   StageClock clk(s);
   Buf core;
   PTTK_TRY(svd_basis(X, m, c, 0.0, core, r, clk, 0, s));
-  return owned_copy(core, m * *r, basis, s);
+  // a copy of its own: cudaFree waits for work that still reads it, and does not for scratch of the pool
+  PTTK_CUDA(cudaMalloc(basis, sizeof(double) * std::max<int64_t>(m * *r, 1)));
+  PTTK_CUDA(cudaMemcpyAsync(*basis, core.p, sizeof(double) * m * *r, cudaMemcpyDeviceToDevice, s));
+  return PTTK_OK;
 }
 
 // One-sided Jacobi on the columns of A (rows x ncols, column-major), in place: on return the
