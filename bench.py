@@ -51,8 +51,8 @@ NOMINAL = {"bf16": 2.25, "tf32": 1.1}
 # DRAM bytes (read + write) of one chain_tc launch of the fast form on this workload, from one
 # ncu capture of the kernel source whose SHA-256 prefix is given: the figure is reported only
 # while the source is unchanged, and null otherwise.
-NCU_TRAFFIC = {"fp16x3": {"src_sha16": "90d8050ec85c5546", "bytes": 1398013160}}
-CHAIN_SRC = os.path.join(ROOT, "paper_2406_06344_gb300", "csrc", "chain_tc.cu")
+NCU_TRAFFIC = {"fp16x3": {"src_sha16": "404ff793a91678bf", "bytes": 1391318016}}
+CHAIN_SRC = [os.path.join(ROOT, "paper_2406_06344_gb300", "csrc", f) for f in ("tcgen05.cuh", "chain_pair.cu")]
 # executed FP64 flops per entry of the FP64 grid kernel (K_nu quadrature + in-tile transform),
 # from ncu instruction counts (DFMA x 2 + DADD + DMUL) on the n = 5 grid of the same workload,
 # tied like NCU_TRAFFIC to the SHA-256 prefix of the kernel sources it was counted on
@@ -167,11 +167,14 @@ def kernel_rooflines(prof, steps, ranks, d, dtheta, n, N, hbm, dfma):
     """A fraction of a measured peak for each kernel group of kernel_ms, from the workload's
     sizes (prof: name -> (total ms, launches) over `steps` bench steps; hbm in GB/s, dfma in
     TFLOP/s):
-    - apply, domain, mode_transform: HBM bytes (FP32 factors; FP32 points; one FP64 and one
-      FP32 grid, each with its D - m1 = 4 strided passes that read and write every entry);
-    - dgemm: FP64 flops of the TT-SVD's projections X <- G_k^T X alone, on the whole unfoldings
-      (the tall steps' X V products and the preconditioned Jacobi's R1^T (P2 V) are not counted;
-      parity sectors execute about a tenth of what is counted);
+    - apply, domain: HBM bytes (FP32 factors; FP32 points);
+    - mode_transform: HBM bytes of one FP64 and one FP32 grid with D - m1 = 4 strided passes that read and
+      write every entry of the whole grid ("bytes", "frac"), and what is executed on the grid folded over
+      the d - 1 dimensions in which the workload's boxes share their centre: the passes on its 2^(1-d) of the
+      entries, and the expansion that reads those and writes all ("bytes_executed", "frac_executed");
+    - dgemm: FP64 flops of the TT-SVD's projections X <- G_k^T X alone, on the whole unfoldings: an
+      equivalent rate ("achieved"; "frac_lower_bound" is its ratio to the peak), no fraction of the peak ("frac" is null):
+      parity sectors execute about a tenth of it;
     - householder, jacobi, theta_core: null, with the reason (their work depends on the QR's
       stopping step, the Jacobi's sweeps, or is latency-bound)."""
     D = 2 * d + dtheta
@@ -200,7 +203,11 @@ def kernel_rooflines(prof, steps, ranks, d, dtheta, n, N, hbm, dfma):
     t_ms, t_cnt = ms_of("mode_transform")
     hbm_entry("mode_transform", steps * 4 * (16.0 + 8.0) * total,
               "per step 4 passes over the FP64 grid (16 B per entry) and 4 over the FP32 grid (8 B), counted on the "
-              "whole grid: the reflection-folded one that is transformed has a quarter of its entries at d = 3")
+              "whole grid; *_executed: 4 passes on the reflection-folded grid and its expansion")
+    if "mode_transform" in out:
+        e, f = out["mode_transform"], 2.0 ** (1 - d)
+        e["bytes_executed"] = steps * (8.0 + 4.0) * total * (4 * 2 * f + f + 1.0)
+        e["frac_executed"] = e["frac"] * e["bytes_executed"] / e["bytes"]
     g_ms, g_cnt = ms_of("dgemm")
     if g_cnt and g_ms > 0:
         proj = 0.0
@@ -210,9 +217,9 @@ def kernel_rooflines(prof, steps, ranks, d, dtheta, n, N, hbm, dfma):
             proj += 2.0 * ranks[k] * c * m
         ach = steps * proj / (g_ms / 1000.0) / 1e12
         out["dgemm"] = {"bound": "alu (FP64 FMA)", "achieved": ach, "peak": dfma, "unit": "TFLOP/s",
-                        "frac_lower_bound": ach / dfma, "launches": g_cnt,
-                        "note": "the TT-SVD projections' flops on the whole unfoldings, nothing else; where parity sectors are "
-                                "found (d = 3: a tenth of these flops is executed) the fraction passes 1"}
+                        "frac": None, "frac_lower_bound": ach / dfma, "launches": g_cnt,
+                        "note": "an equivalent rate, of the TT-SVD projections' flops on the whole unfoldings: parity sectors "
+                                "(d = 3) execute a tenth of them, so its ratio to the peak passes 1 and bounds nothing"}
     for name, why in (("householder", "work depends on the step at which each pivoted QR stops"),
                       ("jacobi", "work depends on the number of sweeps"),
                       ("theta_core", "latency-bound: a few small contractions per theta")):
@@ -834,8 +841,8 @@ def run_extras(torch, P, W, w, tt, X32, Y32, wv, thetas, state, flush, ev, pk, h
     P.grad(tt, th0, Xa, Ya, wa_d, za_d, FAST_FORM)
     P.profile_enable(False)
     adj_ms, _ = P.profile_get("adjoint")
-    src_f = 2.0 * w.n * sum(ranks[i] * ranks[i + 1] for i in range(w.d))
-    adj_flops = 3.0 * src_f * Na
+    # executed: S_2 and Q (r_1 r_2 each), the last step's dot and gbar (r_2 each), the first step forward and back (r_1 each)
+    adj_flops = 4.0 * w.n * (ranks[1] * ranks[2] + ranks[2] + ranks[1]) * Na
     out["adjoint"] = {"workload": "d3 matern-nu TT, N_s=N_t=500k, w,z~N(0,1), loss w^T K~ z",
                       "form": FAST_FORM, "grads_per_s": 1.0 / statistics.median(times),
                       "ms": 1000.0 * statistics.median(times), "dtheta": list(map(float, dth)),
@@ -844,9 +851,8 @@ def run_extras(torch, P, W, w, tt, X32, Y32, wv, thetas, state, flush, ev, pk, h
                       "roofline": {"bound": "alu (FP32 FMA)", "achieved": adj_flops / (adj_ms / 1000.0) / 1e12,
                                    "peak": pk["ffma"], "unit": "TFLOP/s",
                                    "frac": adj_flops / (adj_ms / 1000.0) / 1e12 / pk["ffma"],
-                                   "note": "reverse pass for dL/dX (FP32 SIMT), counted as 3x the source chain's flops; "
-                                           "its last step needs a vector only, so the executed flops are a tenth of it "
-                                           "and the fraction passes 1"}}
+                                   "note": "reverse pass for dL/dX (FP32 SIMT): its executed FP32 multiply-adds; the bases "
+                                           "and the last sums over T_j' are FP64 beside them"}}
 
     # TT-Round (Algorithm 1) of the d = 3 TT: to looser tolerances, and of its sum with itself
     # (ranks doubled), back to 1e-10

@@ -19,7 +19,7 @@
 //    of y_s's index is known, and writes C with exact zeros. (d = 3 boxes shifted along one axis: s = 2.)
 //  - r is formed once per point pair and used for all length scales; the Bessel table is read by Horner's
 //    rule, and the exponential is the table form of fexp.cuh.
-// 12^8 entries, general-nu Matern, FP64: 131.6 -> 21.9 ms.
+// 12^8 entries, general-nu Matern, FP64: 131.6 -> 20.3 ms (FP32 5.9 -> 4.8).
 #include <math.h>
 
 #include <algorithm>
