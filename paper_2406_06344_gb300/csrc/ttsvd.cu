@@ -41,7 +41,6 @@
 namespace pttk {
 namespace {
 
-constexpr int RC = 4096;  // Householder rows per pass of the reflector through shared memory
 constexpr int HU = 8;     // rows per lane per load batch in the Householder passes
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -128,7 +127,7 @@ __global__ void transpose_kernel(const double* __restrict__ X, int64_t m, int64_
 // pivots stood idle (20736 x 3696, 1350 steps: 827 ms; five launches a step 575; now 571). Large batches run three blocks an SM
 // for the FP64 pipe (248832 x 756: 417 -> 402 ms), small ones two, since a barrier costs more with more blocks (3672 x 144: 3.5
 // against 5.1 ms); the line, 8 million elements, lies between 7281 x 729 (23.6 against 27.1 ms) and 10008 x 1728
-// (71.9 against 59.5).
+// (71.9 against 59.5). The former also pass 4096 rows of the reflector at a time instead of 1024 (417 against 438 ms, two blocks).
 struct HHState {
   double tail2;  // ||R22||_F^2 at the stop (0 if every column was factored)
   int k;
@@ -197,7 +196,7 @@ struct QrBatch {
   int count;
 };
 
-template <int PER_SM>
+template <int PER_SM, int RC>  // RC: rows per pass of the reflector through shared memory
 __global__ void __launch_bounds__(256, PER_SM) hh_kernel(QrBatch batch) {
   extern __shared__ unsigned mask[];  // bit p: column p not yet factored; then the columns left before each word
   __shared__ double v[RC];
@@ -336,10 +335,15 @@ __global__ void __launch_bounds__(256, PER_SM) hh_kernel(QrBatch batch) {
       __syncthreads();
     };
     // this block's share of the columns left
-    const int left = N - 1 - j, q_lo = (int)((int64_t)left * cb / CN), q_hi = (int)((int64_t)left * (cb + 1) / CN);
+    // (32 bits: R takes N^2 doubles, so N < 2^18, and there are a few hundred blocks)
+    const unsigned left = (unsigned)(N - 1 - j);
+    const int q_lo = (int)(left * (unsigned)cb / (unsigned)CN), q_hi = (int)(left * (unsigned)(cb + 1) / (unsigned)CN);
+    int p0 = 0, p1 = 0;  // kept for the second pass where there is one set
+    const bool one_set = q_hi - q_lo <= QC;
     for (int c0 = q_lo; c0 < q_hi; c0 += QC) {
       const bool l0 = c0 + warp < q_hi, l1 = c0 + warp + 8 < q_hi;
-      const int p0 = l0 ? column(c0 + warp) : 0, p1 = l1 ? column(c0 + warp + 8) : 0;
+      p0 = l0 ? column(c0 + warp) : 0;
+      p1 = l1 ? column(c0 + warp + 8) : 0;
       const double* ca = A + (int64_t)p0 * M;
       const double* cbp = A + (int64_t)p1 * M;
       double a0 = 0.0, a1 = 0.0;
@@ -373,7 +377,10 @@ __global__ void __launch_bounds__(256, PER_SM) hh_kernel(QrBatch batch) {
     if (!grid_barrier(jb.sync, nblocks)) return;
     for (int c0 = q_lo; c0 < q_hi; c0 += QC) {
       const bool l0 = c0 + warp < q_hi, l1 = c0 + warp + 8 < q_hi;
-      const int p0 = l0 ? column(c0 + warp) : 0, p1 = l1 ? column(c0 + warp + 8) : 0;
+      if (!one_set) {
+        p0 = l0 ? column(c0 + warp) : 0;
+        p1 = l1 ? column(c0 + warp + 8) : 0;
+      }
       // w = tau sum over the row groups
       double w0 = 0.0, w1 = 0.0;
       for (int g = lane; g < RG; g += 32) {
@@ -864,7 +871,7 @@ pttk_status householder_batch(std::vector<Qr>& qr, cudaStream_t s) {
   const size_t smem = (sizeof(unsigned) + sizeof(int)) * (((size_t)nmax + 31) / 32);
   double total = 0.0;
   for (const Qr& q : qr) total += (double)q.M * q.N;
-  auto kfn = total >= 8e6 ? hh_kernel<3> : hh_kernel<2>;
+  auto kfn = total >= 8e6 ? hh_kernel<3, 4096> : hh_kernel<2, 1024>;
   if (smem > 8 * 1024)
     PTTK_CUDA(allow_smem((const void*)kfn));
   int cap = 0;
